@@ -386,7 +386,7 @@ const char *latch_session_last_error(const latch_session *s);
 
 /* ---- Autotuning (tile shapes and path choice, by measurement on this device) ---- */
 typedef struct {
-    int32_t item_kps;           /* extraction: fewest keypoints per block (sets the grid), 1..32 */
+    int32_t item_kps;           /* extraction: fewest keypoints per batch (one block builds their windows), 1..32 */
     int64_t tensor_min_pairs;   /* matching: LATCH_PATH_AUTO uses the tensor cores from nq*nt >= this */
 } latch_tuning;
 
@@ -396,7 +396,7 @@ typedef struct {
     int32_t n_query, n_train;   /* representative matching shape (0: skip the matching tuning) */
 } latch_tune_shape;
 
-/* Measure the candidate extraction work-item sizes and the matching paths on
+/* Measure the candidate extraction batch sizes and the matching paths on
  * synthetic device data of this shape and keep the fastest in the context; results
  * do not change (all candidates compute identical outputs), only speed.  Synchronous;
  * allocates temporary device memory.  `out` (may be NULL) receives the choice. */

@@ -1,6 +1,6 @@
 // Batched extract-then-match (the structure-from-motion shape of Sec. 4-5: many
 // images, each matched against its neighbours).  Enqueues, on one stream:
-//   1. one bucket launch and one persistent extraction launch per 64 images; the
+//   1. one persistent extraction launch per 64 images; the
 //      extraction also writes every descriptor's +-1 E2M1 row for the tensor
 //      matcher (each image's set once, although it serves as query and as train
 //      in several pairs),
@@ -26,7 +26,7 @@ struct BatchPlan {
     std::vector<int64_t> kp0, n, out0;
     int64_t total_kp = 0, total_out = 0;
     int64_t max_tiles = 0;  // query tiles of the largest matching launch
-    size_t ext_bytes = 0, match_bytes = 0;
+    size_t match_bytes = 0;
 };
 
 latch_status plan_batch(latch_context* ctx, const latch_batch_desc* b, BatchPlan* plan) {
@@ -61,7 +61,6 @@ latch_status plan_batch(latch_context* ctx, const latch_batch_desc* b, BatchPlan
         plan->total_out += plan->n[qi];
     }
     if (plan->total_out > 0 && !b->d_matches) return fail(ctx, LATCH_EINVAL, "NULL match output");
-    plan->ext_bytes = (extract_batch_scratch_bytes(b->h_images, plan->n.data(), b->n_images) + 1023) / 1024 * 1024;
     // matching scratch: the largest chunk of pairs
     MatchBatch* mb = new (std::nothrow) MatchBatch;
     if (!mb) return fail(ctx, LATCH_ENOMEM, "host allocation failed");
@@ -108,7 +107,7 @@ extern "C" latch_status latch_reserve_batch(latch_context* ctx, const latch_batc
     if (st != LATCH_OK) return st;
     LATCH_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
     void* p = nullptr;
-    return scratch_reserve(ctx, 3, plan.ext_bytes + plan.match_bytes, &p);
+    return scratch_reserve(ctx, 2, plan.match_bytes, &p);
 }
 
 extern "C" latch_status latch_batch_run(latch_context* ctx, const latch_batch_desc* b, latch_stream_t stream) {
@@ -119,15 +118,14 @@ extern "C" latch_status latch_batch_run(latch_context* ctx, const latch_batch_de
     if (!ctx->has_trip) return fail(ctx, LATCH_EINVAL, "no triplet table: call latch_set_triplets");
     LATCH_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
     void* scratch = nullptr;
-    st = scratch_reserve(ctx, 3, plan.ext_bytes + plan.match_bytes, &scratch);
+    st = scratch_reserve(ctx, 2, plan.match_bytes, &scratch);
     if (st != LATCH_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    uint8_t* base = static_cast<uint8_t*>(scratch);
     cudaEvent_t* ev = (ctx->trace_ev && ctx->trace_n < ctx->trace_cap) ? ctx->trace_ev + 3 * ctx->trace_n++ : nullptr;
     // the extraction also writes the matcher's expanded rows when there is
     // matching to do
     const bool matching = b->n_pairs > 0 && plan.total_out > 0;
-    uint8_t* mbase = base + plan.ext_bytes;
+    uint8_t* mbase = static_cast<uint8_t*>(scratch);
     if (ev) cudaEventRecord(ev[0], s);
     if (matching) {
         // cleared before the extraction, so that nothing sits between the extraction
@@ -141,7 +139,7 @@ extern "C" latch_status latch_batch_run(latch_context* ctx, const latch_batch_de
     if (plan.total_kp > 0) {
         st = cuda_check(ctx,
                         launch_extract_batch(ctx, b->h_images, plan.kp0.data(), plan.n.data(), b->n_images, b->d_kps,
-                                             b->d_desc, base, s, matching ? mbase : nullptr),
+                                             b->d_desc, s, matching ? mbase : nullptr),
                         "batched extraction launch");
         if (st != LATCH_OK) return st;
     }

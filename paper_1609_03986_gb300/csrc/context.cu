@@ -85,21 +85,18 @@ latch_status scratch_reserve(latch_context* ctx, int slot, size_t bytes, void** 
 static latch_status upload_scales(latch_context* ctx, const double* scales, int n) {
     const size_t entries = static_cast<size_t>(n) * kBins * kWinPix;
     int8_t* host = static_cast<int8_t*>(malloc(entries * 2));
-    int16_t* toff = static_cast<int16_t*>(malloc((entries + 16) * sizeof(int16_t)));
+    uint16_t* toff = static_cast<uint16_t*>(malloc(entries * sizeof(uint16_t)));
     if (!host || !toff) {
         free(host);
         free(toff);
         return fail(ctx, LATCH_ENOMEM, "host allocation of offset tables failed");
     }
     build_offset_tables(scales, n, host);
-    const int reach = max_reach(scales, n);
-    const int pitch = extract_tile_pitch(reach);
-    for (size_t i = 0; i < entries; ++i) toff[i] = static_cast<int16_t>(host[2 * i + 1] * pitch + host[2 * i]);
-    for (size_t i = entries; i < entries + 16; ++i) toff[i] = 0;
+    build_tile_offsets(scales, n, host, toff);
     free(host);
-    int16_t* dev = nullptr;
-    cudaError_t e = cudaMalloc(&dev, (entries + 16) * sizeof(int16_t));
-    if (e == cudaSuccess) e = cudaMemcpy(dev, toff, (entries + 16) * sizeof(int16_t), cudaMemcpyHostToDevice);
+    uint16_t* dev = nullptr;
+    cudaError_t e = cudaMalloc(&dev, entries * sizeof(uint16_t));
+    if (e == cudaSuccess) e = cudaMemcpy(dev, toff, entries * sizeof(uint16_t), cudaMemcpyHostToDevice);
     free(toff);
     if (e != cudaSuccess) {
         if (dev) cudaFree(dev);
@@ -116,7 +113,6 @@ static latch_status upload_scales(latch_context* ctx, const double* scales, int 
     ctx->d_tile_offsets = dev;
     ctx->nscales = n;
     for (int i = 0; i < n; ++i) ctx->scales[i] = scales[i];
-    ctx->reach = reach;
     return LATCH_OK;
 }
 
@@ -146,7 +142,7 @@ static latch_status load_triplets(latch_context* ctx, const latch_triplet* t) {
     latch_status st = validate_triplets(ctx, t, ctx->weighted);
     if (st != LATCH_OK) return st;
     memcpy(ctx->h_trip, t, sizeof(ctx->h_trip));
-    build_triplet_offsets(ctx->h_trip, ctx->h_trip_offsets);
+    plan_triplets(ctx->h_trip, ctx->weighted ? kPatchR * 2 + 2 : kPatchR * 2 + 1, &ctx->trip_plan);
     ctx->has_trip = true;
     return LATCH_OK;
 }
@@ -277,6 +273,7 @@ latch_status latch_set_triplets(latch_context* ctx, const latch_triplet* h_tripl
 latch_status latch_set_patch_weights(latch_context* ctx, const uint8_t* h_weights) {
     if (!ctx) return fail(ctx, LATCH_EINVAL, "NULL context");
     if (!h_weights) {
+        if (ctx->weighted && ctx->has_trip) plan_triplets(ctx->h_trip, kPatchR * 2 + 1, &ctx->trip_plan);
         ctx->weighted = false;
         return LATCH_OK;
     }
@@ -285,6 +282,7 @@ latch_status latch_set_patch_weights(latch_context* ctx, const uint8_t* h_weight
         if (st != LATCH_OK) return st;
     }
     for (int i = 0; i < 64; ++i) ctx->patch_weights[i] = h_weights[i];
+    if (!ctx->weighted && ctx->has_trip) plan_triplets(ctx->h_trip, kPatchR * 2 + 2, &ctx->trip_plan);
     ctx->weighted = true;
     return LATCH_OK;
 }
@@ -294,10 +292,9 @@ latch_status latch_reserve(latch_context* ctx, int64_t max_keypoints, int64_t ma
     if (max_keypoints < 0 || max_query < 0 || max_train < 0) return fail(ctx, LATCH_EINVAL, "negative size");
     LATCH_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
     void* p = nullptr;
-    latch_image big{nullptr, 32768, 32768, 32768};
-    latch_status st = scratch_reserve(ctx, 0, extract_scratch_bytes(&big, max_keypoints), &p);
-    if (st == LATCH_OK) st = scratch_reserve(ctx, 1, match_popc_scratch_bytes(ctx, max_query, max_train), &p);
-    if (st == LATCH_OK) st = scratch_reserve(ctx, 2, match_tc_scratch_bytes(ctx, max_query, max_train), &p);
+    // extraction needs none
+    latch_status st = scratch_reserve(ctx, 0, match_popc_scratch_bytes(ctx, max_query, max_train), &p);
+    if (st == LATCH_OK) st = scratch_reserve(ctx, 1, match_tc_scratch_bytes(ctx, max_query, max_train), &p);
     return st;
 }
 
@@ -351,10 +348,7 @@ latch_status latch_extract(latch_context* ctx, const latch_image* img, const lat
     }
     if (!ctx->has_trip) return fail(ctx, LATCH_EINVAL, "no triplet table: pass one or call latch_set_triplets");
     if (n == 0) return LATCH_OK;
-    void* scratch = nullptr;
-    latch_status st = scratch_reserve(ctx, 0, extract_scratch_bytes(img, n), &scratch);
-    if (st != LATCH_OK) return st;
-    return cuda_check(ctx, launch_extract(ctx, img, d_kps, n, d_out, scratch, s), "extract kernel launch");
+    return cuda_check(ctx, launch_extract(ctx, img, d_kps, n, d_out, s), "extract kernel launch");
 }
 
 static latch_status validate_image(latch_context* ctx, const latch_image* img) {
@@ -390,7 +384,7 @@ latch_status latch_detect(latch_context* ctx, const latch_image* img, int32_t th
     LATCH_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
     const double one = 1.0;
     void* scratch = nullptr;
-    st = scratch_reserve(ctx, 4, detect_scratch_bytes(img, &one, 1), &scratch);
+    st = scratch_reserve(ctx, 3, detect_scratch_bytes(img, &one, 1), &scratch);
     if (st != LATCH_OK) return st;
     return cuda_check(ctx,
                       launch_detect(img, &one, &scale_idx, 1, threshold, max_kps, d_kps, d_count, scratch,
@@ -404,14 +398,12 @@ static latch_status detect_levels(latch_context* ctx, const latch_image* img, co
                                   const int32_t* idx, int nlev, int32_t threshold, int32_t max_kps,
                                   latch_keypoint* d_kps, int32_t* d_count, uint8_t* d_desc, cudaStream_t s) {
     void* dscratch = nullptr;
-    void* escratch = nullptr;
-    latch_status st = scratch_reserve(ctx, 4, detect_scratch_bytes(img, scales, nlev), &dscratch);
-    if (st == LATCH_OK && d_desc) st = scratch_reserve(ctx, 0, extract_scratch_bytes(img, max_kps), &escratch);
+    latch_status st = scratch_reserve(ctx, 3, detect_scratch_bytes(img, scales, nlev), &dscratch);
     if (st != LATCH_OK) return st;
     st = cuda_check(ctx, launch_detect(img, scales, idx, nlev, threshold, max_kps, d_kps, d_count, dscratch, s),
                     "detection launch");
     if (st != LATCH_OK || !d_desc) return st;
-    return cuda_check(ctx, launch_extract_dev_count(ctx, img, d_kps, max_kps, d_count, d_desc, escratch, s),
+    return cuda_check(ctx, launch_extract_dev_count(ctx, img, d_kps, max_kps, d_count, d_desc, s),
                       "extraction launch");
 }
 
@@ -471,12 +463,12 @@ latch_status hamming_match(latch_context* ctx, const uint8_t* d_query, int32_t n
     if (path == LATCH_PATH_AUTO) path = choose_match_path(ctx, nq, nt);
     void* scratch = nullptr;
     if (path == LATCH_PATH_TENSOR) {
-        latch_status st = scratch_reserve(ctx, 2, match_tc_scratch_bytes(ctx, nq, nt), &scratch);
+        latch_status st = scratch_reserve(ctx, 1, match_tc_scratch_bytes(ctx, nq, nt), &scratch);
         if (st != LATCH_OK) return st;
         return cuda_check(ctx, launch_match_tc(ctx, d_query, nq, d_train, nt, k, r_milli, d_out, scratch, s),
                           "tensor match launch");
     }
-    latch_status st = scratch_reserve(ctx, 1, match_popc_scratch_bytes(ctx, nq, nt), &scratch);
+    latch_status st = scratch_reserve(ctx, 0, match_popc_scratch_bytes(ctx, nq, nt), &scratch);
     if (st != LATCH_OK) return st;
     return cuda_check(ctx, launch_match_popc(ctx, d_query, nq, d_train, nt, k, r_milli, d_out, scratch, s),
                       "popc match launch");

@@ -1,46 +1,59 @@
 // LATCH descriptor extraction (Sec. 3.1 Eq. 1; Sec. 3.2).
 //
-// 1. sort_count_kernel + sort_scatter_kernel (1024 keypoints per block): counting
-//    sort of the keypoints into 32x32-pixel image cells; the launch's record array
-//    receives one 16-byte record per keypoint (position, output row, offset table,
-//    image), cell by cell.  The
-//    cell grid reaches 128 px beyond every border; keypoints further out have
-//    windows wholly outside the image (the window reaches at most `reach` <= 78
-//    px), whose samples all read 0, so their descriptor is all zeros and is written
-//    here directly.  Keypoints with a scale index outside the scale table also get
-//    zeros and raise the context's device flag.
-// 2. extract_lanes_kernel (one block of 28 warps per SM): the records are taken 32
-//    at a time ("batches", in sort order), one keypoint per lane.  A batch's work
-//    is 64 chunks of 8 triplets; the chunks of all batches are split into G equal
-//    contiguous ranges, range b for block b, so a batch may be shared by two
-//    blocks (each builds its windows and evaluates its own chunks).  The block
-//    is a two-stage pipeline over double-buffered windows:
-//      - 12 builder warps build the 32 windows of batch i: for each run of
-//        keypoints in one image cell, the tile under the cell plus a `reach`
-//        halo is staged into shared memory by one TMA 2-D load (samples outside
-//        the image arrive as 0, the border reading; two tile slots, the next
-//        run's tile requested while the current one is read), and every window
-//        pixel is read from it through the per-(scale, bin) offset table
-//        (nearest pixel; offsets pre-multiplied into tile offsets), in units of
-//        half a window spread over the builder warps, each warp loading the
-//        table words of its next unit while it gathers the current one.  Window
-//        j sits at word 577 j: with an odd stride, the 32 lanes reading the same
-//        word of their windows hit 32 different banks;
-//      - 16 evaluator warps evaluate Eq. 1 on batch i - 1, warp w on chunks 4w ..
-//        4w+3, all 32 lanes on the same triplet at a time (the triplet table is
-//        staged in shared memory: one broadcast load per triplet): a 7-pixel
-//        patch row is two or three words, aligned by a funnel shift; D1 - D2 =
-//        (sum C1^2 - sum C2^2) - 2 (sum A.C1 - sum A.C2) over the 7 rows with
-//        __dp4a, all exact in 32-bit integers.  Each warp writes its bytes of
-//        every lane's descriptor (bit t = bit t % 8 of byte t / 8) and, when
-//        the caller also wants the tensor matcher's input, its 16 bytes of the
-//        expanded row (4-bit value t = E2M1 -1.0 or +1.0 for bit t set or clear).
-//    The stages hand the window buffers over through mbarriers (full: 384
-//    builder arrivals, empty: 16 evaluator arrivals); every wait is bounded.
+// extract_lanes_kernel: one block of 32 warps per SM.  The launch's keypoints are taken
+// in batches of up to 32 in their own order, one keypoint per lane; a batch's work is
+// 64 chunks of 8 triplets.  Whole batches go round the blocks (batch r G + b to block
+// b); the batches of the last, incomplete round are cut into chunk ranges, one per
+// block (every block that evaluates a part of a batch builds the batch's windows).
+// The block is a pipeline:
+//   2 producers    per keypoint one TMA 2-D load of the image tile under its window
+//                  (samples outside the image arrive as 0, the border reading) into a
+//                  byte ring in shared memory; the box is that of the keypoint's scale
+//                  class (at most three box sizes per launch);
+//   12 builders    four groups of three warps, a keypoint per group: the 48x48 window
+//                  through the per-(scale, bin) table of tile offsets (nearest pixel), a
+//                  third of it per warp, into a staging buffer, column of words by column
+//                  of words (word (cx, y) of the window at 48 cx + y);
+//   16 evaluators  first copy the batch's staged words into tensor memory, window j in
+//                  TMEM lane j of every lane quarter, which frees the staging buffer for
+//                  the next batch; then evaluate Eq. 1, all 32 lanes on the same triplet:
+//                  a patch is two or three columns of words, so as many 8-row TMEM loads
+//                  bring it, its rows are aligned by funnel shifts, and D1 - D2 =
+//                  (sum C1^2 - sum C2^2) - 2 (sum A.C1 - sum A.C2) by __dp4a, all exact in
+//                  32-bit integers.  A ballot gives a triplet's bit of all 32 keypoints;
+//                  the bits are transposed and leave as whole rows, with the tensor
+//                  matcher's expanded row when it is wanted.
+//
+// Why tensor memory: every lane needs 52.5 window words per triplet.  From shared memory
+// (128 bytes per clock per SM) that alone is 840 wavefronts per keypoint, and it bound the
+// kernel; tensor memory delivers 128 bytes per clock to each of the four SM partitions,
+// so the loads no longer limit and shared memory holds tiles instead of two buffers of
+// windows.  512 columns hold 504 of a window's 576 words.  As all four quarters hold the
+// same keypoints, each keeps another part of the window, from another byte of a word on,
+// and a triplet is evaluated in a quarter that holds its patches, where most of them start
+// at a word and need no alignment (25 of 42 shifts are left on the seeded table).  The
+// evaluation is bound by instruction issue (about 125 instructions per triplet, 56 of
+// them dot products) shared with the builders.
+//
+// Why a tile per keypoint: no sort by image cell is needed (it cost a memset and two
+// launches in front of the extraction), builders need no barrier between keypoints, and at
+// the density of photographs (about two keypoints per 32x32 cell) a cell's tile is as
+// many bytes per keypoint as the keypoint's own.
+//
+// Keypoints whose window misses the image read only zeros, and so get the zero
+// descriptor; one with a scale index outside the scale table is moved far outside for
+// the same result and raises the context's device flag.
+//
+// Measured (GB300, whole calls back to back; before: windows in shared memory, cell sort):
+// 257 keypoints of 321x243 46.9 -> 18.4 us, 2,000 of 640x480 44.1 -> 22.7 us, 10,000 of
+// 1920x1080 91.4 -> 52.8 us, the same weighted 189 -> 134 us.
 #include <cuda.h>
 
+#include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <new>
+#include <type_traits>
 
 #include "internal.h"
 #include "sm103.h"
@@ -51,285 +64,80 @@ namespace {
 
 using namespace sm103;
 
-constexpr int kCell = 32;
-constexpr int kMargin = 128;            // cell grid reaches this far beyond each border
-constexpr int kBuildWarps = 12;         // window builders (4, 8, 16 measured slower)
-constexpr int kComputeWarps = 16;       // Eq. 1 evaluators (4 chunks each per batch)
-constexpr int kBuildThreads = 32 * kBuildWarps;
-constexpr int kComputeThreads = 32 * kComputeWarps;
-constexpr int kThreads = kBuildThreads + kComputeThreads;  // 896
-constexpr int kRowWords = 12;           // 48 bytes per window row
-constexpr int kWinWords = kWinPix / 4;  // 576 words per window
-constexpr int kLaneWords = kWinWords + 1;          // window stride: odd, so a warp's same-offset loads hit 32 banks
+constexpr int kGroups = 4;              // builder groups, one keypoint each at a time
+constexpr int kGroupWarps = 3;
+constexpr int kBuildWarps = kGroups * kGroupWarps;  // warps 0-11
+constexpr int kProducers = 2;           // warps 12, 13 (14, 15 idle: register splits go by four warps)
+constexpr int kEvalWarp0 = 16;          // warps 16-31 evaluate
+constexpr int kEvalWarps = 16;
+constexpr int kEvalThreads = 32 * kEvalWarps;
+constexpr int kThreads = 32 * (kEvalWarp0 + kEvalWarps);
 constexpr int kBatch = 32;              // keypoints per batch, one per lane
 constexpr int kChunks = kBits / 8;      // chunks of 8 triplets per batch
-constexpr int kSortThreads = 256;
-constexpr int kSortKps = 1024;          // keypoints per sorting block (4 per thread)
+constexpr int kWordCols = kWin / 4;     // 12 columns of words in a window
+constexpr int kBlockWords = 32;         // a builder unit: 4 word columns x 8 rows, one word per lane
+constexpr int kBlocks = kWordCols * kWin / kBlockWords;    // 18 units per window
+constexpr int kWarpBlocks = kBlocks / kGroupWarps;         // 6 per builder warp
+constexpr int kTmemCols = 512;
+constexpr int kTmLast = kTmemCols - 8;  // last column an 8-column load may start at
+constexpr int kStageWords = kWordCols * kWin + 1;          // odd: the 32 lanes' copies hit 32 banks
+constexpr int kExtRows = kWin - 42;     // the rows quarter 0 lacks, kept in shared memory too
+constexpr int kExtWords = kExtRows * kWordCols + 1;        // odd, as above
+constexpr int kOutWords = 33;           // descriptor word w of lane l at 33 w + l
+constexpr int kSlots = 8;               // tiles in flight at most, per producer
+constexpr int kClasses = 3;             // tile box sizes per launch
+// registers per thread after the split (1024 threads x 64 at launch)
+constexpr int kBuildRegs = 48, kProducerRegs = 24, kEvalRegs = 80;
+static_assert(kGroupWarps * 4 == kWordCols && kWarpBlocks * 8 == kWin, "a builder warp takes four word columns");
+static_assert(kBuildWarps * kBuildRegs + 4 * kProducerRegs + kEvalWarps * kEvalRegs <= 32 * 64, "register split");
 
-struct CellGrid {
-    int gx, gy;  // cells in x / y (including the margins)
-    int width, height;
+// What each TMEM lane quarter holds of a window (576 words do not fit its 512 columns):
+// `nc` columns of words from byte column `b0` on, rows r0 .. r0 + nr - 1, word (k, r) at
+// column k nr + r.  Each quarter lacks a different margin and starts at a different byte
+// of a word, and a triplet goes to a quarter that holds its three patches, of these to
+// one in which most of them start at a word (plan_triplets).  Quarter 0 takes those that
+// fit none, with rows 42..47 from shared memory.
+struct Quarter {
+    int32_t b0, nc, r0, nr;
 };
-
-// Cell of a keypoint: >= 0, -1 (window wholly outside: zero descriptor), -2 (bad scale).
-__device__ __forceinline__ int cell_of(const latch_keypoint& kp, int nscales, const CellGrid& g) {
-    if (kp.scale_idx >= nscales) return -2;
-    const int64_t x = static_cast<int64_t>(kp.x) + kMargin, y = static_cast<int64_t>(kp.y) + kMargin;
-    if (x < 0 || y < 0 || x >= static_cast<int64_t>(g.width) + 2 * kMargin ||
-        y >= static_cast<int64_t>(g.height) + 2 * kMargin)
-        return -1;
-    return static_cast<int>(y / kCell) * g.gx + static_cast<int>(x / kCell);
+constexpr int kQuarters = 4;
+__host__ __device__ constexpr Quarter quarter_of(int q) {
+    return q == 0 ? Quarter{0, 12, 0, 42} : q == 1 ? Quarter{1, 12, 6, 42} : q == 2 ? Quarter{2, 10, 0, 48} : Quarter{7, 10, 0, 48};
 }
 
-struct TileGeom {
-    int tw, th;      // staged tile (bytes per row, rows)
-    int mx, my;      // tile origin relative to the cell origin (negative)
+struct TileClass {
+    int32_t reach;      // |offset| of every window sample is at most this
+    int32_t tw, th;     // box: bytes per row, rows
 };
 
 // Per-launch description of a batch of images (kernel parameters).
 template <int NI>
 struct ExtractParams {
-    CUtensorMap map[NI];  // one TMA map per image
-    CellGrid grid[NI];
-    int32_t kp0[NI];      // first keypoint of image i in the concatenated keypoint array
-    int32_t n[NI];        // keypoints of image i
-    int32_t cell0[NI];    // first entry of image i in the global cell-count scratch
-    int32_t blk0[NI];     // first sorting block of image i (ceil(n / kSortKps) blocks each)
-    int32_t count;        // images in this launch
+    CUtensorMap map[NI * kClasses];  // map of image i and class c at i * kClasses + c
+    const int32_t* n_dev;    // single-image launches: the keypoint count on the device (n is its bound), or NULL
+    int32_t n;               // keypoints in this launch
+    int32_t row0;            // row of the launch's first keypoint in the keypoint and output arrays
+    int32_t min_batch;       // fewest keypoints per batch (latch_tuning.item_kps)
     int32_t nscales;
-    TileGeom tg;
-    const int32_t* n_dev;  // single-image launches: the keypoint count on the device (n[0] is its bound), or NULL
+    int32_t count;           // images in this launch
+    TileClass cls[kClasses];
+    int8_t cls_of[LATCH_MAX_SCALES];
+    int32_t width[NI], height[NI];
+    int32_t first[NI];       // keypoints of the launch before image i
 };
 
-// Keypoints of image `img` in this launch.
-template <int NI>
-__device__ __forceinline__ int keypoints_of(const ExtractParams<NI>& prm, int img) {
-    const int n = prm.n[img];
-    if (!prm.n_dev) return n;
-    const int d = *prm.n_dev;
-    return d < n ? (d > 0 ? d : 0) : n;
-}
-
-// Sorted keypoint record: x, y, output row (the keypoint's index), table (scale *
-// 32 + bin) | launch-local image << 16.
-__device__ __forceinline__ int4 kp_record(const latch_keypoint& kp, int row, int img) {
-    return make_int4(kp.x, kp.y, row, (kp.scale_idx * kBins + (kp.angle_bin & (kBins - 1))) | (img << 16));
-}
-
-// Image of sorting block `blk` (largest i with blk0[i] <= blk).
-template <int NI>
-__device__ __forceinline__ int image_of_block(const ExtractParams<NI>& prm, int blk) {
-    int lo = 0, hi = prm.count - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (prm.blk0[mid] <= blk) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-// Sorting, pass 1 (kSortKps keypoints of one image per block): the cell of every
-// keypoint; a keypoint with a cell takes its rank in the cell from an atomic on the
-// cell's count (order of arrival), one without gets its zero descriptor here.  The
-// last block of an image to finish turns the image's counts into exclusive starts.
-// Scratch zeroed by the host: img_tot / img_done, the cell counts.
-template <int NI>
-__global__ void __launch_bounds__(kSortThreads) sort_count_kernel(
-    const __grid_constant__ ExtractParams<NI> prm, const latch_keypoint* __restrict__ kps, int* __restrict__ cells,
-    int* __restrict__ rank, int* __restrict__ img_tot, int* __restrict__ img_done, uint4* __restrict__ out,
-    uint4* __restrict__ exp_out, uint32_t* __restrict__ flags) {
-    __shared__ int s_part[kSortThreads / 32];
-    __shared__ int s_flag;
-    griddep_wait();
-    griddep_launch_dependents();
-    const int img = image_of_block(prm, blockIdx.x);
-    const CellGrid g = prm.grid[img];
-    const int n = keypoints_of(prm, img), kp0 = prm.kp0[img];
-    int* cnt = cells + prm.cell0[img];
-    const int i0 = (blockIdx.x - prm.blk0[img]) * kSortKps + threadIdx.x;
-    // all loads first, then the atomics
-    latch_keypoint kp[kSortKps / kSortThreads];
-#pragma unroll
-    for (int q = 0; q < kSortKps / kSortThreads; ++q)
-        if (i0 + q * kSortThreads < n) kp[q] = kps[kp0 + i0 + q * kSortThreads];
-    int valid = 0;
-    bool bad = false;
-#pragma unroll
-    for (int q = 0; q < kSortKps / kSortThreads; ++q) {
-        const int i = i0 + q * kSortThreads;
-        const int c = i < n ? cell_of(kp[q], prm.nscales, g) : -3;
-        if (c >= 0) {
-            rank[kp0 + i] = atomicAdd(&cnt[c], 1);
-            ++valid;
-        } else if (c > -3) {
-            const uint4 z = make_uint4(0, 0, 0, 0);
-            uint4* d = out + static_cast<size_t>(kp0 + i) * 4;
-            d[0] = z;
-            d[1] = z;
-            d[2] = z;
-            d[3] = z;
-            if (exp_out) {  // the expanded row of the zero descriptor: every value +1.0
-                uint4* x = exp_out + static_cast<size_t>(kp0 + i) * (kExpRowBytes / 16);
-                const uint4 one = expand_word_e2m1(0u);
-                for (int u = 0; u < kExpRowBytes / 16; ++u) x[u] = one;
-            }
-            bad |= (c == -2);
-        }
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    valid = __reduce_add_sync(0xffffffffu, static_cast<uint32_t>(valid));
-    if (lane == 0) s_part[warp] = valid;
-    if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flags, kFlagBadScale);
-    if (threadIdx.x == 0) {
-        int v = 0;
-        for (int w = 0; w < kSortThreads / 32; ++w) v += s_part[w];
-        atomicAdd(&img_tot[img], v);
-        // release: the block's count increments (ordered before this by the barrier
-        // above) and its total, before its arrival
-        __threadfence();
-        const int nblk = (prm.n[img] + kSortKps - 1) / kSortKps;  // every launched block of the image arrives
-        s_flag = atomicAdd(&img_done[img], 1) == nblk - 1;
-    }
-    __syncthreads();
-    if (!s_flag) return;
-    // ---- last block of the image: exclusive starts of its cells, in place, in
-    // tiles of 8 cells per thread (eight independent loads in flight) ----
-    __threadfence();
-    const int ncell = g.gx * g.gy;
-    int carry = 0;
-    for (int tb = 0; tb < ncell; tb += 8 * kSortThreads) {
-        const int c0 = tb + 8 * threadIdx.x;
-        int v[8];
-        int sum = 0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            v[q] = c0 + q < ncell ? __ldcg(&cnt[c0 + q]) : 0;
-            sum += v[q];
-        }
-        int incl = sum;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int x = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += x;
-        }
-        __syncthreads();  // s_part free (its previous readers are done)
-        if (lane == 31) s_part[warp] = incl;
-        __syncthreads();
-        int run = carry + incl - sum, tile_total = 0;
-        for (int w = 0; w < kSortThreads / 32; ++w) {
-            const int x = s_part[w];
-            if (w < warp) run += x;
-            tile_total += x;
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-            if (c0 + q < ncell) {
-                cnt[c0 + q] = run;
-                run += v[q];
-            }
-        carry += tile_total;
-    }
-}
-
-// Sorting, pass 2 (same blocks): each keypoint with a cell writes its record at
-// image base + cell start + rank; the records of all images are contiguous, image
-// by image (base = the totals of the earlier images).  Block 0 sets counters[0] =
-// the launch's number of records.
-template <int NI>
-__global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(
-    const __grid_constant__ ExtractParams<NI> prm, const latch_keypoint* __restrict__ kps,
-    const int* __restrict__ cells, const int* __restrict__ rank, const int* __restrict__ img_tot,
-    int* __restrict__ counters, int4* __restrict__ recs) {
-    __shared__ int s_base;
-    griddep_wait();
-    griddep_launch_dependents();
-    const int img = image_of_block(prm, blockIdx.x);
-    const CellGrid g = prm.grid[img];
-    const int n = keypoints_of(prm, img), kp0 = prm.kp0[img];
-    const int* start = cells + prm.cell0[img];
-    const int i0 = (blockIdx.x - prm.blk0[img]) * kSortKps + threadIdx.x;
-    latch_keypoint kp[kSortKps / kSortThreads];
-#pragma unroll
-    for (int q = 0; q < kSortKps / kSortThreads; ++q)
-        if (i0 + q * kSortThreads < n) kp[q] = kps[kp0 + i0 + q * kSortThreads];
-    if (threadIdx.x < 32) {  // at most 64 images
-        const int lane = threadIdx.x;
-        const int a = lane < prm.count ? img_tot[lane] : 0;
-        const int b = lane + 32 < prm.count ? img_tot[lane + 32] : 0;
-        const int before = (lane < img ? a : 0) + (lane + 32 < img ? b : 0);
-        const int base = __reduce_add_sync(0xffffffffu, static_cast<uint32_t>(before));
-        const int total = __reduce_add_sync(0xffffffffu, static_cast<uint32_t>(a + b));
-        if (lane == 0) {
-            s_base = base;
-            if (blockIdx.x == 0) counters[0] = total;
-        }
-    }
-    __syncthreads();
-    const int base = s_base;
-#pragma unroll
-    for (int q = 0; q < kSortKps / kSortThreads; ++q) {
-        const int i = i0 + q * kSortThreads;
-        const int c = i < n ? cell_of(kp[q], prm.nscales, g) : -3;
-        if (c >= 0) recs[base + start[c] + rank[kp0 + i]] = kp_record(kp[q], kp0 + i, img);
-    }
-}
-
-// Tile key of a record: launch-local image, cell row and column (the record's
-// keypoint has a cell, so x + kMargin and y + kMargin are >= 0).
-__device__ __forceinline__ int tile_key(const int4& r) {
-    return ((r.w >> 16) << 22) | (((r.y + kMargin) / kCell) << 11) | ((r.x + kMargin) / kCell);
-}
-
-// Window words of every triplet's three patches (top-left word of the 7x7 patch
-// in a 48x48 window of 12-word rows) and their byte shifts: x = A | C1 << 16,
-// y = C2 | shift A << 16 | shift C1 << 18 | shift C2 << 20.
+// The triplets as the evaluators read them (from constant memory: the index is the
+// same for a whole warp, so the fields are unpacked once per warp), quarter by quarter
+// and class by class: a word per patch (anchor, companions), bits 0-4 the byte shift
+// times 8 (what a funnel shift takes), bits 16-24 the TMEM column of the patch's first
+// word; bits 5-13 of the anchor's: the triplet's index.  A triplet's class has bit p set
+// when patch p does not start at a word (its rows must be aligned); class 8 (quarter 0):
+// it lies past the quarter's rows or three word columns from its first would not fit.
+constexpr int kTripClasses = 9;
 struct LaneTriplets {
-    uint2 e[kBits];
+    uint32_t e[3][kBits];
+    int16_t start[kQuarters][kTripClasses + 1];  // first entry of each class
 };
-
-// One patch row: the 7 bytes at byte `sh` of word p[0] onwards, as two words whose
-// last byte is junk (the third word is read only when the bytes reach into it).
-__device__ __forceinline__ void patch_row(const uint32_t* p, uint32_t sh, uint32_t& lo, uint32_t& hi) {
-    const uint32_t w0 = p[0], w1 = p[1];
-    const uint32_t w2 = sh >= 2 ? p[2] : 0u;
-    lo = __funnelshift_r(w0, w1, 8 * sh);
-    hi = __funnelshift_r(w1, w2, 8 * sh);
-}
-
-// Bit i of the result: Eq. 1 for triplet 8 c + i of the window at `wl` (`trip`:
-// the LaneTriplets entries, in shared memory: one broadcast load per triplet).
-__device__ __forceinline__ uint32_t eval_chunk(const uint2* trip, const uint32_t* wl, int c) {
-    uint32_t byte = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const uint2 e = trip[8 * c + i];
-        const uint32_t* pa = wl + (e.x & 0xffffu);
-        const uint32_t* p1 = wl + (e.x >> 16);
-        const uint32_t* p2 = wl + (e.y & 0xffffu);
-        const uint32_t sa = (e.y >> 16) & 3u, s1 = (e.y >> 18) & 3u, s2 = (e.y >> 20) & 3u;
-        uint32_t sa1 = 0, sa2 = 0, s11 = 0, s22 = 0;
-#pragma unroll
-        for (int rr = 0; rr < 2 * kPatchR + 1; ++rr) {
-            uint32_t a0, a1, c0, c1, d0, d1;
-            patch_row(pa + rr * kRowWords, sa, a0, a1);
-            patch_row(p1 + rr * kRowWords, s1, c0, c1);
-            patch_row(p2 + rr * kRowWords, s2, d0, d1);
-            c1 &= 0x00ffffffu;  // pixel 8 of the run is not in the patch (A's is multiplied by 0)
-            d1 &= 0x00ffffffu;
-            sa1 = __dp4a(a0, c0, sa1);
-            sa1 = __dp4a(a1, c1, sa1);
-            sa2 = __dp4a(a0, d0, sa2);
-            sa2 = __dp4a(a1, d1, sa2);
-            s11 = __dp4a(c0, c0, s11);
-            s11 = __dp4a(c1, c1, s11);
-            s22 = __dp4a(d0, d0, s22);
-            s22 = __dp4a(d1, d1, s22);
-        }
-        // D1 - D2 = sum C1^2 - sum C2^2 - 2 (sum A.C1 - sum A.C2)
-        const int diff =
-            (static_cast<int>(s11) - static_cast<int>(s22)) - 2 * (static_cast<int>(sa1) - static_cast<int>(sa2));
-        byte |= (diff > 0 ? 1u : 0u) << i;
-    }
-    return byte;
-}
 
 // Weights of the 8x8 patch pixels (row-major), a kernel parameter: with the pixel
 // loops unrolled, every weight is a constant-bank operand of its multiply-add.
@@ -337,292 +145,642 @@ struct PatchWeights {
     int32_t w[64];
 };
 
-// One 8-pixel patch row: the 8 bytes at byte `sh` of word p[0] onwards, as two words.
-__device__ __forceinline__ void patch_row8(const uint32_t* p, uint32_t sh, uint32_t& lo, uint32_t& hi) {
-    const uint32_t w0 = p[0], w1 = p[1];
-    const uint32_t w2 = sh != 0 ? p[2] : 0u;
-    lo = __funnelshift_r(w0, w1, 8 * sh);
-    hi = __funnelshift_r(w1, w2, 8 * sh);
-}
+// The block's share of the launch as items: a batch and its chunk range [ca, cb).
+struct Item {
+    int32_t kp0, nk;  // first keypoint in the launch, keypoints
+    int32_t ca, cb;
+};
 
-// Eq. 1 with weighted 8x8 patches (Sec. 3.2, weighing pixels in LATCH patches) for
-// triplets 8 c .. 8 c + 7: D1 - D2 = sum w (C1 - C2)(C1 + C2 - 2 A), exact in int32
-// (|w (C1 - C2)(C1 + C2 - 2 A)| <= 255 * 255^2 per pixel, 64 pixels).
-__device__ __forceinline__ uint32_t eval_chunk_weighted(const uint2* trip, const uint32_t* wl, int c,
-                                                        const PatchWeights& pw) {
-    uint32_t byte = 0;
-#pragma unroll 1
-    for (int i = 0; i < 8; ++i) {
-        const uint2 e = trip[8 * c + i];
-        const uint32_t* pa = wl + (e.x & 0xffffu);
-        const uint32_t* p1 = wl + (e.x >> 16);
-        const uint32_t* p2 = wl + (e.y & 0xffffu);
-        const uint32_t sa = (e.y >> 16) & 3u, s1 = (e.y >> 18) & 3u, s2 = (e.y >> 20) & 3u;
-        int acc = 0;
-#pragma unroll
-        for (int rr = 0; rr < 8; ++rr) {
-            uint32_t a[2], c1[2], c2[2];
-            patch_row8(pa + rr * kRowWords, sa, a[0], a[1]);
-            patch_row8(p1 + rr * kRowWords, s1, c1[0], c1[1]);
-            patch_row8(p2 + rr * kRowWords, s2, c2[0], c2[1]);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int av = static_cast<int>((a[j >> 2] >> (8 * (j & 3))) & 0xffu);
-                const int cv = static_cast<int>((c1[j >> 2] >> (8 * (j & 3))) & 0xffu);
-                const int dv = static_cast<int>((c2[j >> 2] >> (8 * (j & 3))) & 0xffu);
-                acc += pw.w[rr * 8 + j] * ((cv - dv) * (cv + dv - 2 * av));
-            }
+struct Work {
+    int32_t n, bs;       // keypoints of the launch, per batch
+    int32_t rounds, items;
+    int32_t tail0;       // first batch of the incomplete round
+    int32_t u0, u1;      // the block's chunk range in it
+    __device__ __forceinline__ Item item(int i) const {
+        Item it;
+        int batch;
+        if (i < rounds) {
+            batch = i * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x);
+            it.ca = 0;
+            it.cb = kChunks;
+        } else {
+            const int t = u0 / kChunks + (i - rounds);
+            batch = tail0 + t;
+            it.ca = max(u0, t * kChunks) - t * kChunks;
+            it.cb = min(u1, (t + 1) * kChunks) - t * kChunks;
         }
-        byte |= (acc > 0 ? 1u : 0u) << i;
+        it.kp0 = batch * bs;
+        it.nk = min(bs, n - it.kp0);
+        return it;
     }
-    return byte;
+};
+
+// Batch size: 32 (every lane busy) once the launch gives each block a batch or more.
+// Below that a block builds bs windows for the chunks it evaluates of them, about
+// kBuildCost bs + kEvalCost n / (G bs) clocks, least at bs = sqrt(kEvalCost n /
+// (kBuildCost G)).
+template <int NI>
+__device__ __forceinline__ Work plan_work(const ExtractParams<NI>& prm, int n) {
+    constexpr float kCostRatio = 60.0f;  // evaluation of a batch (16k clocks) / building a window (270 clocks)
+    Work w;
+    const uint32_t G = gridDim.x, b = blockIdx.x;
+    w.n = n;
+    w.bs = min(kBatch, max(prm.min_batch, static_cast<int>(sqrtf(kCostRatio * static_cast<float>(w.n) / static_cast<float>(G)))));
+    const int nb = (w.n + w.bs - 1) / w.bs;
+    w.rounds = static_cast<int>(static_cast<uint32_t>(nb) / G);
+    w.tail0 = w.rounds * static_cast<int>(G);
+    const uint32_t u = static_cast<uint32_t>(nb - w.tail0) * kChunks;  // below 64 G: the products fit 32 bits
+    w.u0 = static_cast<int>(b * u / G);
+    w.u1 = static_cast<int>((b + 1) * u / G);
+    w.items = w.rounds + (w.u1 > w.u0 ? (w.u1 - 1) / kChunks - w.u0 / kChunks + 1 : 0);
+    return w;
 }
 
 struct LanesSmem {  // static part
-    uint2 trip[kBits];                // LaneTriplets
-    int4 rec[2][kBatch];              // builders: the batch's records
-    int32_t row[2][kBatch];           // output row of each lane's keypoint
-    uint64_t tile_bar[2], full[2], empty[2];
-    uint32_t runs[2];
+    uint32_t bits[2][kBits];                  // entry p of the triplet list: bit j = keypoint j's (double-buffered)
+    uint32_t out[kEvalWarps * kOutWords];     // descriptor words of the item
+    uint16_t entry[kBits];                    // list entry of each triplet
+    uint32_t base[kProducers * kSlots];       // ring byte of the tile's sample at offset (-reach, -reach)
+    uint64_t full[kProducers * kSlots], empty[kProducers * kSlots];  // tiles
+    uint64_t staged, copied;                  // window staging buffer
+    Work work;                                // the evaluators' copy (it would take registers)
+    uint32_t tmem;
     int abort;
 };
 
-// Block b takes chunks [b U / G, (b+1) U / G) of the U = 64 * ceil(V / 32) chunks
-// of the launch's V records (cell-sorted), batch by batch.  Warps 0-11 build the
-// windows of batch i into buffer i % 2 while warps 12-27 evaluate batch i - 1.
+constexpr size_t kFixedSmem = 128 + (static_cast<size_t>(kBatch) * kStageWords + 2 * kBatch * kExtWords) * 4;
+constexpr int kRingBytes = static_cast<int>((227 * 1024 - sizeof(LanesSmem) - kFixedSmem) / 128 * 128);
+constexpr size_t kDynSmem = kFixedSmem + kRingBytes;
+
+// ---- evaluation --------------------------------------------------------------------
+
+// Requests the word columns of a patch (its word `f`), 8 rows each, from the lane quarter
+// at `tm` (whose column bits are zero) with `nr` rows per word column: two of a patch of
+// at most 8 columns that starts at a word, else three.  kClamp: the third may lie past the
+// last column (the patch does not need it then).
+template <bool kThree, bool kClamp = false>
+__device__ __forceinline__ void request(uint32_t (&w)[3][8], uint32_t f, uint32_t tm, uint32_t nr) {
+    const uint32_t a = (f >> 16) + tm;
+    tmem_ld_32x32b_x8(a, w[0]);
+    tmem_ld_32x32b_x8(a + nr, w[1]);
+    if constexpr (kThree) tmem_ld_32x32b_x8(kClamp ? min(a + 2 * nr, tm + kTmLast) : a + 2 * nr, w[2]);
+}
+
+// After tmem_ld_wait(): pins the loaded registers behind the wait (the compiler may move
+// plain arithmetic above it).
+template <bool kThree, int kRows>
+__device__ __forceinline__ void arrive(uint32_t (&w)[3][8]) {
+#pragma unroll
+    for (int k = 0; k < (kThree ? 3 : 2); ++k)
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) asm volatile("" : "+r"(w[k][r]));
+}
+
+// Aligns the rows: w[0][r] = pixels 0..3 and w[1][r] = pixels 4..7 of the patch row.
+template <int kRows>
+__device__ __forceinline__ void align(uint32_t (&w)[3][8], uint32_t f) {
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {  // (a funnel shift takes 5 bits of f)
+        w[0][r] = __funnelshift_r(w[0][r], w[1][r], f);
+        w[1][r] = __funnelshift_r(w[1][r], w[2][r], f);
+    }
+}
+
+// The rows that quarter 0 lacks, from `ext` (the lane's rows 42..47, 12 words each).  All
+// rows are loaded and the missing ones selected: a branch per row would cost a load's
+// latency each.
+template <int kRows>
+__device__ __forceinline__ void fill(uint32_t (&w)[3][8], uint32_t f, const uint32_t* ext) {
+    constexpr int nr = quarter_of(0).nr;
+    const int col = static_cast<int>(f >> 16), cx = col / nr, y0 = col - cx * nr;
+    if (y0 + kRows <= nr) return;
+    const uint32_t* x = ext + cx;
+    const int third = cx + 2 < kWordCols ? 2 : 1;
+#pragma unroll
+    for (int r = 1; r < kRows; ++r) {
+        const int row = y0 + r - nr;
+        const uint32_t* xr = x + max(row, 0) * kWordCols;
+        const uint32_t v0 = xr[0], v1 = xr[1], v2 = xr[third];
+        w[0][r] = row >= 0 ? v0 : w[0][r];
+        w[1][r] = row >= 0 ? v1 : w[1][r];
+        w[2][r] = row >= 0 ? v2 : w[2][r];
+    }
+}
+
+// The words of one triplet (LaneTriplets).
+struct Words {
+    uint32_t a, c1, c2;
+    __device__ __forceinline__ int index() const { return static_cast<int>((a >> 5) & 511u); }
+};
+__device__ __forceinline__ Words words_of(const LaneTriplets& tt, int p) {
+    return Words{tt.e[0][p], tt.e[1][p], tt.e[2][p]};
+}
+
+// sum A.C and sum C^2 over the 7 patch rows (pixel 8 of a row is not in the patch: masked
+// in C, and A's is multiplied by it).
+__device__ __forceinline__ void dot7(const uint32_t (&a)[3][8], const uint32_t (&c)[3][8], uint32_t& ac, uint32_t& cc) {
+    ac = 0;
+    cc = 0;
+#pragma unroll
+    for (int r = 0; r < 7; ++r) {
+        const uint32_t hi = c[1][r] & 0x00ffffffu;
+        ac = __dp4a(a[0][r], c[0][r], ac);
+        cc = __dp4a(c[0][r], c[0][r], cc);
+        ac = __dp4a(a[1][r], hi, ac);
+        cc = __dp4a(hi, hi, cc);
+    }
+}
+
+// D1 > D2 from the sums: D1 - D2 = sum C1^2 - sum C2^2 - 2 (sum A.C1 - sum A.C2).
+__device__ __forceinline__ bool farther(uint32_t ac1, uint32_t cc1, uint32_t ac2, uint32_t cc2) {
+    return (static_cast<int>(cc1) - static_cast<int>(cc2)) - 2 * (static_cast<int>(ac1) - static_cast<int>(ac2)) > 0;
+}
+
+// Eq. 1 for every fourth entry (those = `mine` mod 4) of one class' list entries [lo, hi):
+// bits[p] = the bits of all lanes' keypoints.  The next triplet's first companion is
+// requested under the second half of this one, its anchor at the end of it (the registers
+// are free then): the other warps of the partition cover what is left of the wait.
+template <int kClass>
+__device__ __forceinline__ void eval_class(const LaneTriplets& tt, int lo, int hi, int mine, uint32_t tm, uint32_t nr,
+                                           uint32_t* bits, int lane) {
+    constexpr bool kA = kClass & 1, k1 = kClass & 2, k2 = kClass & 4;
+    int p = lo + ((mine - lo) & 3);
+    if (p >= hi) return;
+    const int first = p;
+    uint32_t a[3][8], c[3][8], d[3][8];
+    Words f = words_of(tt, p);
+    request<k1>(c, f.c1, tm, nr);
+    request<kA>(a, f.a, tm, nr);
+#pragma unroll 1
+    for (; p < hi; p += 4) {
+        const Words g = words_of(tt, p + 4 < hi ? p + 4 : first);
+        tmem_ld_wait();
+        arrive<k1, 7>(c);
+        arrive<kA, 7>(a);
+        request<k2>(d, f.c2, tm, nr);
+        if constexpr (kA) align<7>(a, f.a);
+        if constexpr (k1) align<7>(c, f.c1);
+        uint32_t ac1, cc1, ac2, cc2;
+        dot7(a, c, ac1, cc1);
+        tmem_ld_wait();
+        arrive<k2, 7>(d);
+        request<k1>(c, g.c1, tm, nr);
+        if constexpr (k2) align<7>(d, f.c2);
+        dot7(a, d, ac2, cc2);
+        request<kA>(a, g.a, tm, nr);
+        const uint32_t b = __ballot_sync(0xffffffffu, farther(ac1, cc1, ac2, cc2));
+        if (lane == 0) bits[p] = b;
+        f = g;
+    }
+    tmem_ld_wait();
+}
+
+// Eq. 1 for one triplet of any class (kExt: class 8), not pipelined.
+template <bool kExt>
+__device__ __forceinline__ bool eval_any(const Words& f, uint32_t tm, uint32_t nr, const uint32_t* ext) {
+    uint32_t a[3][8], c[3][8], d[3][8];
+    request<true, true>(a, f.a, tm, nr);
+    request<true, true>(c, f.c1, tm, nr);
+    tmem_ld_wait();
+    arrive<true, 7>(a);
+    arrive<true, 7>(c);
+    request<true, true>(d, f.c2, tm, nr);
+    if constexpr (kExt) {
+        fill<7>(a, f.a, ext);
+        fill<7>(c, f.c1, ext);
+    }
+    align<7>(a, f.a);
+    align<7>(c, f.c1);
+    uint32_t ac1, cc1, ac2, cc2;
+    dot7(a, c, ac1, cc1);
+    tmem_ld_wait();
+    arrive<true, 7>(d);
+    if constexpr (kExt) fill<7>(d, f.c2, ext);
+    align<7>(d, f.c2);
+    dot7(a, d, ac2, cc2);
+    return farther(ac1, cc1, ac2, cc2);
+}
+
+// Eq. 1 with weighted 8x8 patches (Sec. 3.2, weighing pixels in LATCH patches):
+// D1 - D2 = sum w (C1 - C2)(C1 + C2 - 2 A), exact in int32 (|w (C1 - C2)(C1 + C2 - 2 A)|
+// <= 255 * 255^2 per pixel, 64 pixels).
+template <bool kExt>
+__device__ __forceinline__ bool eval_triplet_weighted(const Words& f, uint32_t tm, uint32_t nr, const uint32_t* ext,
+                                                      const PatchWeights& pw) {
+    uint32_t a[3][8], c[3][8], d[3][8];
+    request<true, true>(a, f.a, tm, nr);
+    request<true, true>(c, f.c1, tm, nr);
+    tmem_ld_wait();
+    arrive<true, 8>(a);
+    arrive<true, 8>(c);
+    if constexpr (kExt) {
+        fill<8>(a, f.a, ext);
+        fill<8>(c, f.c1, ext);
+    }
+    align<8>(a, f.a);
+    align<8>(c, f.c1);
+    request<true, true>(d, f.c2, tm, nr);
+    tmem_ld_wait();
+    arrive<true, 8>(d);
+    if constexpr (kExt) fill<8>(d, f.c2, ext);
+    align<8>(d, f.c2);
+    int acc = 0;
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const uint32_t sel = 0x4440u | static_cast<uint32_t>(j & 3);
+            const int av = static_cast<int>(__byte_perm(a[j >> 2][r], 0u, sel));
+            const int cv = static_cast<int>(__byte_perm(c[j >> 2][r], 0u, sel));
+            const int dv = static_cast<int>(__byte_perm(d[j >> 2][r], 0u, sel));
+            acc += pw.w[r * 8 + j] * ((cv - dv) * (cv + dv - 2 * av));
+        }
+    return acc > 0;
+}
+
+// The quarter's triplets [t0, t1) one at a time: weighted patches, a part of the chunks,
+// and class 8.
+template <bool kWeighted>
+__device__ __forceinline__ void eval_entries(const LaneTriplets& tt, const PatchWeights& pw, int lo, int hi, int ext0,
+                                             int mine, int t0, int t1, uint32_t tm, uint32_t nr, const uint32_t* ext,
+                                             uint32_t* bits, int lane) {
+#pragma unroll 1
+    for (int p = lo + ((mine - lo) & 3); p < hi; p += 4) {
+        const Words f = words_of(tt, p);
+        const int t = f.index();
+        if (t < t0 || t >= t1) continue;
+        bool bit;
+        if (p < ext0) {
+            if constexpr (kWeighted)
+                bit = eval_triplet_weighted<false>(f, tm, nr, ext, pw);
+            else
+                bit = eval_any<false>(f, tm, nr, ext);
+        } else {
+            if constexpr (kWeighted)
+                bit = eval_triplet_weighted<true>(f, tm, nr, ext, pw);
+            else
+                bit = eval_any<true>(f, tm, nr, ext);
+        }
+        const uint32_t b = __ballot_sync(0xffffffffu, bit);
+        if (lane == 0) bits[p] = b;
+    }
+}
+
+// The warp's share (`mine` of 4) of the quarter's triplets [t0, t1).
+template <bool kWeighted>
+__device__ __forceinline__ void eval_quarter(const LaneTriplets& tt, const PatchWeights& pw, int quarter, int mine,
+                                             int t0, int t1, uint32_t tm, uint32_t nr, const uint32_t* ext,
+                                             uint32_t* bits, int lane) {
+    const int16_t* start = tt.start[quarter];
+    int lo = start[0];
+    if (!kWeighted && t1 - t0 == kBits) {
+        eval_class<0>(tt, start[0], start[1], mine, tm, nr, bits, lane);
+        eval_class<1>(tt, start[1], start[2], mine, tm, nr, bits, lane);
+        eval_class<2>(tt, start[2], start[3], mine, tm, nr, bits, lane);
+        eval_class<3>(tt, start[3], start[4], mine, tm, nr, bits, lane);
+        eval_class<4>(tt, start[4], start[5], mine, tm, nr, bits, lane);
+        eval_class<5>(tt, start[5], start[6], mine, tm, nr, bits, lane);
+        eval_class<6>(tt, start[6], start[7], mine, tm, nr, bits, lane);
+        eval_class<7>(tt, start[7], start[8], mine, tm, nr, bits, lane);
+        lo = start[8];
+    }
+    eval_entries<kWeighted>(tt, pw, lo, start[9], start[8], mine, t0, t1, tm, nr, ext, bits, lane);
+}
+
+// Copies kRows rows (from row r of the quarter on) of the lane's staged window into the
+// quarter, along the word columns; each word is joined from two of the window's.
+template <int kRows>
+__device__ __forceinline__ void copy_rows(const uint32_t* window, const Quarter& Q, int r, uint32_t tm) {
+    static_assert(kRows == 12 || kRows == 6, "row split");
+    const int c0 = Q.b0 >> 2;
+    const uint32_t sh = 8u * static_cast<uint32_t>(Q.b0 & 3);
+    const uint32_t* src = window + c0 * kWin + Q.r0 + r;
+    uint32_t w[kRows];
+#pragma unroll
+    for (int q = 0; q < kRows; ++q) w[q] = src[q];
+#pragma unroll 2
+    for (int k = 0; k < Q.nc; ++k) {
+        // (past the last word column: bytes that no patch uses)
+        src += c0 + k + 1 < kWordCols ? kWin : 0;
+        uint32_t v[kRows];
+#pragma unroll
+        for (int q = 0; q < kRows; ++q) {
+            const uint32_t n = src[q];
+            v[q] = __funnelshift_r(w[q], n, sh);
+            w[q] = n;
+        }
+        const uint32_t to = tm + static_cast<uint32_t>(k * Q.nr + r);
+        if constexpr (kRows == 12) {
+            tmem_st_32x32b_x8(to, v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]);
+            tmem_st_32x32b_x4(to + 8, v[8], v[9], v[10], v[11]);
+        } else {
+            tmem_st_32x32b_x4(to, v[0], v[1], v[2], v[3]);
+            tmem_st_32x32b_x2(to + 4, v[4], v[5]);
+        }
+    }
+}
+
 template <int NI, bool kWeighted>
 __global__ void __launch_bounds__(kThreads, 1) extract_lanes_kernel(
     const __grid_constant__ ExtractParams<NI> prm, const __grid_constant__ LaneTriplets tt,
-    const __grid_constant__ PatchWeights pw,
-    const int4* __restrict__ recs, const int* __restrict__ counters, const int16_t* __restrict__ toff,
-    uint8_t* __restrict__ out, uint8_t* __restrict__ exp_out, uint32_t* __restrict__ flags) {
+    const __grid_constant__ PatchWeights pw, const latch_keypoint* __restrict__ kps,
+    const uint2* __restrict__ toff, uint8_t* __restrict__ out, uint8_t* __restrict__ exp_out,
+    uint32_t* __restrict__ flags) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ LanesSmem S;
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
-    const TileGeom tg = prm.tg;
-    const int tile_bytes = (tg.tw * tg.th + 127) / 128 * 128;
-    uint32_t* s_win0 = reinterpret_cast<uint32_t*>(smem);  // [2][32][kLaneWords]
-    uint8_t* s_tile0 = smem + 2 * static_cast<size_t>(kBatch) * kLaneWords * 4;  // [2][tile_bytes]
-    griddep_wait();
-    griddep_launch_dependents();
-    const int nrec = counters[0];
-    if (nrec <= 0) return;
-    const int64_t units = static_cast<int64_t>((nrec + kBatch - 1) / kBatch) * kChunks;
-    const int64_t u0 = static_cast<int64_t>(blockIdx.x) * units / gridDim.x;
-    const int64_t u1 = static_cast<int64_t>(blockIdx.x + 1) * units / gridDim.x;
-    if (u0 >= u1) return;
-    const int bfirst = static_cast<int>(u0 / kChunks), blast = static_cast<int>((u1 - 1) / kChunks);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint8_t* ring = smem_raw + (-smem_u32(smem_raw) & 127u);
+    uint32_t* s_stage = reinterpret_cast<uint32_t*>(ring + kRingBytes);  // [kBatch][kStageWords]
+    uint32_t* s_ext = s_stage + kBatch * kStageWords;                        // [2][kBatch][kExtWords]
+    const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     volatile int* abort = &S.abort;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < 2; ++s) {
-            mbar_init(&S.tile_bar[s], 1);
-            mbar_init(&S.full[s], kBuildThreads);
-            mbar_init(&S.empty[s], kComputeWarps);
+        for (int s = 0; s < kProducers * kSlots; ++s) {
+            mbar_init(&S.full[s], 1);
+            mbar_init(&S.empty[s], kGroupWarps);
         }
+        mbar_init(&S.staged, kBuildWarps);
+        mbar_init(&S.copied, kEvalWarps);
         S.abort = 0;
         fence_mbar_init();
     }
-    if (threadIdx.x < kBatch && kBatch * bfirst + lane < nrec) S.rec[0][lane] = recs[kBatch * bfirst + lane];
-    for (int t = threadIdx.x; t < kBits; t += kThreads) S.trip[t] = tt.e[t];
-    __syncthreads();  // the last block-wide barrier: the two roles meet only at mbarriers from here on
+    if (warp == kEvalWarp0) {
+        tmem_alloc(&S.tmem, kTmemCols);
+        tc_fence_before();
+    }
+    if (warp == kBuildWarps && lane < min(kClasses * prm.count, 32)) prefetch_tmap(&prm.map[lane]);
+    __syncthreads();  // the last block-wide barrier: the roles meet only at mbarriers from here on
+    tc_fence_after();
+    // everything above and, in the evaluators, the triplet list touches only parameters,
+    // shared memory and TMEM: it runs under the previous kernel's end
+    auto start = [&]() {
+        Work w;
+        if (!prm.n_dev) w = plan_work(prm, prm.n);
+        griddep_wait();
+        griddep_launch_dependents();
+        if (prm.n_dev) w = plan_work(prm, min(prm.n, max(0, *prm.n_dev)));
+        return w;
+    };
 
     if (warp < kBuildWarps) {
-        // ================= builders (named barrier 1) =================
-        const int tb = threadIdx.x;
-        auto issue_tile = [&](int slot, int key) {  // thread 0; the slot is free
-            const int img = key >> 22;
-            const int tx = (key & 2047) * kCell - kMargin + tg.mx;
-            const int ty = ((key >> 11) & 2047) * kCell - kMargin + tg.my;
-            mbar_arrive_expect_tx(&S.tile_bar[slot], static_cast<uint32_t>(tg.tw * tg.th));
-            tma_load_2d(s_tile0 + slot * tile_bytes, &prm.map[img], tx, ty, &S.tile_bar[slot]);
+        // ================= builders =================
+        set_max_regs_dec<kBuildRegs>();
+        const Work work = start();
+        const int g = warp / kGroupWarps, wi = warp - g * kGroupWarps;
+        // the group takes the keypoints whose sequence number in the block is g mod kGroups
+        const latch_keypoint* kp_launch = kps + prm.row0;
+        // offset tables of an item's keypoints, lane = keypoint
+        auto load_tables = [&](const Item& it) {
+            if (lane >= it.nk) return 0u;
+            const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(kp_launch + it.kp0 + lane) + 2);
+            const uint32_t s = (w >> 8) & 0xffu;
+            return (s < static_cast<uint32_t>(prm.nscales) ? s * kBins : 0u) + (w & (kBins - 1));
         };
-        int g = 0, issued = 1;  // runs started / tiles requested (run r uses slot r % 2)
-        if (tb == 0) issue_tile(0, tile_key(S.rec[0][0]));
+        uint2 tab[kWarpBlocks];
+        const uint2* tab_lane = toff + wi * kBlockWords + lane;  // the lane's word of unit q: kGroupWarps q units on
+        // the lane's word of unit q: word column 4 wi + lane % 4, row 8 q + lane / 4
+        const int cx = 4 * wi + (lane & 3), yl = lane >> 2;
+        const uint32_t ring_addr = smem_u32(ring);
+        const uint32_t stage_addr = smem_u32(s_stage) + 4u * static_cast<uint32_t>(cx * kWin + yl);
+        const uint32_t ext_addr = smem_u32(s_ext) + 4u * static_cast<uint32_t>((yl - (8 - kExtRows)) * kWordCols + cx);
+        int seq0 = 0;        // sequence number of the item's first keypoint
         bool ok = true;
-        for (int bt = bfirst; bt <= blast && ok; ++bt) {
-            const int i = bt - bfirst, buf = i & 1;
-            const int4* rec = S.rec[buf];
-            const int nk = nrec - kBatch * bt < kBatch ? nrec - kBatch * bt : kBatch;
-            uint32_t* win = s_win0 + buf * (kBatch * kLaneWords);
-            // the next batch's first record (for its first tile) and all its records
-            int4 next_first = make_int4(0, 0, 0, 0);
-            if (bt < blast) {
-                if (tb == 0) next_first = recs[kBatch * (bt + 1)];
-                if (warp == kBuildWarps - 1 && kBatch * (bt + 1) + lane < nrec)
-                    cp_async_16(&S.rec[buf ^ 1][lane], recs + kBatch * (bt + 1) + lane);
+        bool primed = false; // tab holds the group's next keypoint
+        Item it = work.item(0);
+        uint32_t tables = work.items > 0 ? load_tables(it) : 0u;
+        for (int i = 0; i < work.items && ok; ++i) {
+            // the next item's tables are on their way while this one is built
+            const Item ni = work.item(i + 1);
+            const uint32_t next_tables = i + 1 < work.items ? load_tables(ni) : 0u;
+            const int j0 = (g - seq0) & (kGroups - 1);
+            if (!primed && j0 < it.nk) {
+                const uint32_t t = __shfl_sync(0xffffffffu, tables, j0);
+#pragma unroll
+                for (int q = 0; q < kWarpBlocks; ++q)
+                    tab[q] = __ldg(tab_lane + t * (kBlocks * kBlockWords) + q * (kGroupWarps * kBlockWords));
+                primed = true;
             }
-            if (warp == 0) {  // runs of keypoints in one cell
-                const int key = lane < nk ? tile_key(rec[lane]) : -1;
-                const int prev = __shfl_up_sync(0xffffffffu, key, 1);
-                const uint32_t starts = __ballot_sync(0xffffffffu, lane < nk && (lane == 0 || key != prev));
-                if (lane == 0) S.runs[buf] = starts;
-            }
-            // window buffer `buf` is free once the evaluators are done with batch i - 2
-            if (i >= 2) ok = mbar_wait(&S.empty[buf], ((i >> 1) - 1) & 1, abort);
-            if (ok && tb < nk) S.row[buf][tb] = rec[tb].z;
-            ok = bar_and<1, kBuildThreads>(ok);
-            if (!ok) break;
-            // Each run of keypoints in one cell is built as units of half a window
-            // (288 words, 9 per lane) spread over the builder warps: unit u of a run is
-            // keypoint j0 + u / 2, half u % 2, and warp w takes units w, w + 12, ..., so
-            // the keypoints of a run are gathered in parallel.  A warp loads the
-            // offset-table words of its next unit (in this run or a later one of the
-            // batch) into B while it gathers the current unit from A.
-            constexpr int kHalves = 2;
-            constexpr int kUnitWords = kWinWords / kHalves;     // 288
-            constexpr int kLaneUnitWords = kUnitWords / 32;     // 9
-            // this warp's unit after unit u of run [j0, j1) (later runs: `rest`), as
-            // keypoint << 1 | half, or -1
-            auto next_unit = [&](int j0, int j1, int u, uint32_t rest) -> int {
-                if (u + kBuildWarps < (j1 - j0) * kHalves) {
-                    const int v = u + kBuildWarps;
-                    return ((j0 + v / kHalves) << 1) | (v % kHalves);
-                }
-                while (rest) {
-                    const int a0 = __ffs(rest) - 1;
-                    rest &= rest - 1;
-                    const int a1 = rest ? __ffs(rest) - 1 : nk;
-                    if (warp < (a1 - a0) * kHalves) return ((a0 + warp / kHalves) << 1) | (warp % kHalves);
-                }
-                return -1;
-            };
-            auto load_unit = [&](int code, uint2 (&e)[kLaneUnitWords]) {
-                if (code < 0) return;
-                const uint2* tab = reinterpret_cast<const uint2*>(toff + static_cast<size_t>(rec[code >> 1].w & 0xffff) * kWinPix) +
-                                   (code & 1) * kUnitWords + lane;
-#pragma unroll
-                for (int q = 0; q < kLaneUnitWords; ++q) e[q] = __ldg(tab + 32 * q);
-            };
-            uint32_t rem = S.runs[buf];
-            uint2 A[kLaneUnitWords], B[kLaneUnitWords];
-            load_unit(next_unit(0, 0, -kBuildWarps, rem), A);
-            while (rem) {
-                const int j0 = __ffs(rem) - 1;
-                rem &= rem - 1;
-                const int j1 = rem ? __ffs(rem) - 1 : nk;
-                const int slot = g & 1;
-                const int key = tile_key(rec[j0]);
-                // request the following run's tile into the other slot (its last
-                // reader, run g - 1, finished at the barrier that ended it)
-                if (tb == 0) {
-                    const int nkey = rem ? tile_key(rec[__ffs(rem) - 1]) : bt < blast ? tile_key(next_first) : -1;
-                    if (nkey >= 0) {
-                        issue_tile(slot ^ 1, nkey);
-                        ++issued;
-                    }
-                }
-                const bool tok = mbar_wait(&S.tile_bar[slot], (g >> 1) & 1, abort);
-                if (tok) {
-                    const uint8_t* tile = s_tile0 + slot * tile_bytes;
-                    const int ox = (key & 2047) * kCell - kMargin + tg.mx;
-                    const int oy = ((key >> 11) & 2047) * kCell - kMargin + tg.my;
-                    for (int u = warp; u < (j1 - j0) * kHalves; u += kBuildWarps) {
-                        load_unit(next_unit(j0, j1, u, rem), B);  // lands during this unit's gathers
-                        const int j = j0 + u / kHalves, half = u % kHalves;
-                        const int4 r = rec[j];
-                        const uint8_t* t = tile + (r.y - oy) * tg.tw + (r.x - ox);
-                        uint32_t* w = win + j * kLaneWords + half * kUnitWords + lane;
-#pragma unroll
-                        for (int q = 0; q < kLaneUnitWords; ++q) {
-                            const uint32_t b0 = t[static_cast<int16_t>(A[q].x & 0xffffu)];
-                            const uint32_t b1 = t[static_cast<int16_t>(A[q].x >> 16)];
-                            const uint32_t b2 = t[static_cast<int16_t>(A[q].y & 0xffffu)];
-                            const uint32_t b3 = t[static_cast<int16_t>(A[q].y >> 16)];
-                            w[32 * q] = b0 | (b1 << 8) | (b2 << 16) | (b3 << 24);
-                        }
-#pragma unroll
-                        for (int q = 0; q < kLaneUnitWords; ++q) A[q] = B[q];
-                    }
-                }
-                if (j1 == nk && warp == kBuildWarps - 1) cp_async_wait_all();
-                ok = bar_and<1, kBuildThreads>(tok);  // the run's tile slot is free after it
+            // the staging buffer is free once the evaluators have copied item i - 1
+            if (i > 0) ok = mbar_wait_sleep<200>(&S.copied, (i - 1) & 1, abort);
+            for (int j = j0; ok && j < it.nk; j += kGroups) {
+                // the group's next keypoint: in this item or the first in the next one
+                const bool same = j + kGroups < it.nk;
+                const int nj = same ? j + kGroups : (g - seq0 - it.nk) & (kGroups - 1);
+                const bool more = same || (i + 1 < work.items && nj < ni.nk);
+                const uint32_t nt = __shfl_sync(0xffffffffu, same ? tables : next_tables, nj);
+                const int seq = (seq0 + j) / kProducers, slot = (g & (kProducers - 1)) * kSlots + seq % kSlots;
+                ok = mbar_wait_sleep<64>(&S.full[slot], static_cast<uint32_t>(seq / kSlots) & 1u, abort);
                 if (!ok) break;
-                ++g;
+                const uint32_t t = ring_addr + S.base[slot];
+                const uint32_t to = stage_addr + 4u * kStageWords * static_cast<uint32_t>(j);
+                const uint2* next_tab = tab_lane + nt * (kBlocks * kBlockWords);
+#pragma unroll
+                for (int q = 0; q < kWarpBlocks; ++q) {
+                    const uint2 e = tab[q];
+                    const uint32_t b0 = lds_u8(t + (e.x & 0xffffu)), b1 = lds_u8(t + (e.x >> 16));
+                    const uint32_t b2 = lds_u8(t + (e.y & 0xffffu)), b3 = lds_u8(t + (e.y >> 16));
+                    // lands during the rest of this keypoint (the last keypoint's is not used)
+                    tab[q] = __ldg(next_tab + q * (kGroupWarps * kBlockWords));
+                    const uint32_t v = __byte_perm(__byte_perm(b0, b1, 0x0040), __byte_perm(b2, b3, 0x0040), 0x5410);
+                    sts_u32(to + 32u * q, v);
+                    if (q == kWarpBlocks - 1 && yl >= 8 - kExtRows)  // rows 42..47
+                        sts_u32(ext_addr + 4u * kExtWords * static_cast<uint32_t>((i & 1) * kBatch + j), v);
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&S.empty[slot]);  // the tile is free for this warp
+                primed = more;
             }
-            // batch i's windows are complete (the barrier above ordered all builders' stores)
-            if (ok) mbar_arrive(&S.full[buf]);
+            __syncwarp();
+            if (ok && lane == 0) mbar_arrive(&S.staged);
+            seq0 += it.nk;
+            it = ni;
+            tables = next_tables;
+        }
+        if (!ok && lane == 0) atomicOr(flags, kFlagTimeout);
+        return;
+    }
+
+    if (warp < kEvalWarp0) {
+        set_max_regs_dec<kProducerRegs>();
+        const int pw = warp - kBuildWarps;
+        if (pw >= kProducers) return;
+        const Work work = start();
+        // ================= producers: tiles into byte rings =================
+        // Producer pw takes the keypoints whose sequence number in the block is pw mod
+        // kProducers, and has its part of the ring and of the slots.
+        // tiles [oldest, seq) are in the ring in order; lane s remembers where slot s's tile
+        // starts.  [head, limit): the free bytes behind the latest tile, up to the oldest
+        // tile or the ring's end.  The warp's own chain of instructions is what limits how
+        // fast it can issue, so everything per keypoint is prepared 32 at a time.
+        constexpr int kPart = kRingBytes / kProducers / 128 * 128;
+        uint8_t* part = ring + pw * kPart;
+        uint64_t *full = S.full + pw * kSlots, *empty = S.empty + pw * kSlots;
+        int head = 0, limit = kPart, my_start = 0, oldest = 0, seq = 0, seq0 = 0;
+        bool ok = true;
+        for (int i = 0; i < work.items && ok; ++i) {
+            const Item it = work.item(i);
+            int bytes = 0, tx = 0, ty = 0, ox = 0;
+            const CUtensorMap* map = nullptr;
+            if (lane < it.nk) {
+                const int k = it.kp0 + lane;
+                const latch_keypoint kp = kps[prm.row0 + k];
+                int lo = 0, hi = prm.count - 1;  // image: largest i with first[i] <= k
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (prm.first[mid] <= k) lo = mid; else hi = mid - 1;
+                }
+                const bool bad = kp.scale_idx >= prm.nscales;
+                if (bad) atomicOr(flags, kFlagBadScale);
+                const int c = prm.cls_of[bad ? 0 : kp.scale_idx];
+                const int r = prm.cls[c].reach;
+                // a keypoint 1024 pixels outside sees as little of the image as any further out
+                const int x = bad ? -1024 : min(max(kp.x, -1024), prm.width[lo] + 1024);
+                const int y = min(max(kp.y, -1024), prm.height[lo] + 1024);
+                tx = (x - r) & ~15;  // TMA: the first byte of a row is a multiple of 16
+                ty = y - r;
+                ox = x - r - tx;
+                bytes = prm.cls[c].tw * prm.cls[c].th;
+                map = &prm.map[lo * kClasses + c];
+            }
+            const int j0 = (pw - seq0) & (kProducers - 1);
+            int size = __shfl_sync(0xffffffffu, bytes, j0);
+            for (int j = j0; j < it.nk; j += kProducers) {
+                size = (size + 127) & ~127;
+                while (seq - oldest == kSlots || head + size > limit) {
+                    if (seq - oldest < kSlots && limit == kPart && oldest < seq) {
+                        head = 0;  // go round: free up to the oldest tile
+                        limit = __shfl_sync(0xffffffffu, my_start, oldest % kSlots);
+                        continue;
+                    }
+                    ok = __all_sync(0xffffffffu, mbar_wait_sleep<20>(&empty[oldest % kSlots],
+                                                                     static_cast<uint32_t>(oldest / kSlots) & 1u, abort));
+                    if (!ok) break;
+                    if (++oldest == seq) {
+                        head = 0;
+                        limit = kPart;
+                    } else {
+                        const int tail = __shfl_sync(0xffffffffu, my_start, oldest % kSlots);
+                        limit = tail >= head ? tail : kPart;
+                    }
+                }
+                if (!ok) break;
+                const int slot = seq % kSlots;
+                if (lane == slot) my_start = head;
+                if (lane == j) {
+                    S.base[pw * kSlots + slot] = static_cast<uint32_t>(pw * kPart + head + ox);
+                    mbar_arrive_expect_tx(&full[slot], static_cast<uint32_t>(bytes));
+                    tma_load_2d(part + head, map, tx, ty, &full[slot]);
+                }
+                head += size;
+                ++seq;
+                size = __shfl_sync(0xffffffffu, bytes, j + kProducers);
+            }
+            seq0 += it.nk;
         }
         if (!ok) {  // let the copies in flight land before the block's memory is released
-            if (tb == 0) {
+            if (lane == 0) {
                 atomicOr(flags, kFlagTimeout);
                 const uint64_t t0 = globaltimer();
-                for (int r = g; r < issued; ++r)
-                    while (!mbar_try_wait(&S.tile_bar[r & 1], (r >> 1) & 1) && globaltimer() - t0 < 200000000ull) {
+                for (int s = seq > kSlots ? seq - kSlots : 0; s < seq; ++s)
+                    while (!mbar_try_wait(&full[s % kSlots], static_cast<uint32_t>(s / kSlots) & 1u) &&
+                           globaltimer() - t0 < 200000000ull) {
                     }
             }
-            if (warp == kBuildWarps - 1) cp_async_wait_all();
+            __syncwarp();
         }
         return;
     }
 
-    // ================= evaluators (named barrier 2) =================
-    const int cw = warp - kBuildWarps;
-    const int ct = cw * 32 + lane;  // 0 .. kComputeThreads - 1
-    for (int bt = bfirst; bt <= blast; ++bt) {
-        const int i = bt - bfirst, buf = i & 1;
-        const int nk = nrec - kBatch * bt < kBatch ? nrec - kBatch * bt : kBatch;
-        const int64_t bu = static_cast<int64_t>(bt) * kChunks;  // the batch's first chunk
-        const int ca = static_cast<int>((u0 > bu ? u0 : bu) - bu);
-        const int cb = static_cast<int>((u1 < bu + kChunks ? u1 : bu + kChunks) - bu);
-        // the evaluator warps agree on the outcome of the wait, so that all of them
-        // reach the barriers below or none does
-        const bool got = mbar_wait(&S.full[buf], (i >> 1) & 1, abort);
-        if (!bar_and<2, kComputeThreads>(got)) {
-            if (!got && lane == 0) atomicOr(flags, kFlagTimeout);
-            return;
-        }
-        // ---- Eq. 1: this warp's chunks [wa, wb), lane = keypoint ----
-        const int n = cb - ca;
-        const int wa = ca + cw * n / kComputeWarps, wb = ca + (cw + 1) * n / kComputeWarps;
-        uint32_t* wbuf = s_win0 + buf * (kBatch * kLaneWords);
-        const uint32_t* wl = wbuf + lane * kLaneWords;
-        uint32_t v = 0;  // byte c - wa: chunk c
-#pragma unroll 1
-        for (int c = wa; c < wb; ++c) {
-            if constexpr (kWeighted)
-                v |= eval_chunk_weighted(S.trip, wl, c, pw) << (8 * (c - wa));
+    // ================= evaluators =================
+    set_max_regs_inc<kEvalRegs>();
+    const int cw = warp - kEvalWarp0;
+    const int ct = cw * 32 + lane;  // 0 .. kEvalThreads - 1
+    const int quarter = warp & 3;   // TMEM lane quarter this warp may access
+    // uniform over the warp, and known to be (shuffles), as TMEM addresses have to be
+    const uint32_t tm = __shfl_sync(0xffffffffu, S.tmem, 0) + (static_cast<uint32_t>(quarter * 32) << 16);
+    const Quarter Q = quarter_of(quarter);
+    const uint32_t nr = static_cast<uint32_t>(Q.nr);
+    {   // the triplet list's positions (only the evaluators use them)
+        S.entry[(tt.e[0][ct] >> 5) & 511u] = static_cast<uint16_t>(ct);
+        const Work w = start();
+        if (ct == 0) S.work = w;
+        bar_sync_id(5, kEvalThreads);
+    }
+    bool dead = false;  // after a failed wait: barriers without work, so that every warp reaches them
+    for (int i = 0; i < S.work.items; ++i) {
+        const Item it = S.work.item(i);
+        if (!dead) dead = !__all_sync(0xffffffffu, mbar_wait_sleep<100>(&S.staged, i & 1, abort));
+        if (!dead) {
+            // copy the staged windows (lane = keypoint) into this quarter, 12 rows per warp
+            tc_fence_after();
+            const int r0 = 12 * (cw >> 2);
+            if (r0 + 12 <= Q.nr)
+                copy_rows<12>(s_stage + lane * kStageWords, Q, r0, tm);
             else
-                v |= eval_chunk(S.trip, wl, c) << (8 * (c - wa));
-        }
-        if (n == kChunks) {
-            // ---- the whole batch is this block's: warp cw holds bytes [4 cw, 4 cw + 4)
-            // of every lane's descriptor.  Once every warp is done with the windows,
-            // the words are staged in the buffer's head (transposed: word cw of lane r at
-            // [cw][r]) and whole rows leave as 16-byte stores: 4 threads per 64-byte
-            // descriptor, 16 per 256-byte expanded row ----
-            bar_sync<2, kComputeThreads>();
-            wbuf[cw * kBatch + lane] = v;
-            bar_sync<2, kComputeThreads>();
-            if (ct < 4 * nk) {
-                const int r = ct >> 2, q = ct & 3;
-                const uint4 d = make_uint4(wbuf[(4 * q) * kBatch + r], wbuf[(4 * q + 1) * kBatch + r],
-                                           wbuf[(4 * q + 2) * kBatch + r], wbuf[(4 * q + 3) * kBatch + r]);
-                reinterpret_cast<uint4*>(out + static_cast<size_t>(S.row[buf][r]) * kDescBytes)[q] = d;
-            }
-            if (exp_out && ct < 16 * nk) {
-                const int r = ct >> 4, w = ct & 15;
-                reinterpret_cast<uint4*>(exp_out + static_cast<size_t>(S.row[buf][r]) * kExpRowBytes)[w] =
-                    expand_word_e2m1(wbuf[w * kBatch + r]);
-            }
+                copy_rows<6>(s_stage + lane * kStageWords, Q, r0, tm);
+            tmem_st_wait();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&S.empty[buf]);  // the windows and rows are free again
-            continue;
+            if (lane == 0) mbar_arrive(&S.copied);
         }
-        // ---- a batch shared with the neighbouring block: this block's bytes [ca, cb)
-        // only, descriptor bytes [wa, wb) and expanded bytes [8 wa, 8 wb) per warp ----
-        const int32_t row = S.row[buf][lane];
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&S.empty[buf]);  // the windows and rows are free again
-        if (wb == wa || lane >= nk) continue;
-        uint8_t* d = out + static_cast<size_t>(row) * kDescBytes;
-        for (int c = wa; c < wb; ++c) {
-            const uint32_t byte = (v >> (8 * (c - wa))) & 0xffu;
-            d[c] = static_cast<uint8_t>(byte);
-            if (exp_out)
-                reinterpret_cast<uint32_t*>(exp_out + static_cast<size_t>(row) * kExpRowBytes)[c] =
-                    expand_byte_e2m1(byte);
+        tc_fence_before();
+        bar_sync_id(1 + quarter, 128);
+        tc_fence_after();
+        uint32_t* bits = S.bits[i & 1];
+        const int n = it.cb - it.ca;
+        if (!dead) {
+            // ---- Eq. 1: this warp's share of the quarter's triplets in the chunks [ca, cb) ----
+            const uint32_t* ext = s_ext + (i & 1) * (kBatch * kExtWords) + lane * kExtWords;
+            const int t0 = __shfl_sync(0xffffffffu, 8 * it.ca, 0), t1 = __shfl_sync(0xffffffffu, 8 * it.cb, 0);
+            eval_quarter<kWeighted>(tt, pw, quarter, (warp >> 2) & 3, t0, t1, tm, nr, ext, bits, lane);
         }
+        tc_fence_before();
+        // all bits of the item are there, and (the buffers alternate) everybody is done with
+        // the other buffer
+        bar_sync_id(5, kEvalThreads);
+        tc_fence_after();
+        uint32_t* so = S.out;
+        {   // warp cw: triplets 32 cw .. 32 cw + 31 of every keypoint, transposed: lane = keypoint
+            uint32_t v = bits[S.entry[32 * cw + lane]];
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) {
+                constexpr uint32_t kMask[5] = {0x55555555u, 0x33333333u, 0x0f0f0f0fu, 0x00ff00ffu, 0x0000ffffu};
+                const uint32_t m = kMask[o == 16 ? 4 : o == 8 ? 3 : o == 4 ? 2 : o == 2 ? 1 : 0];
+                const uint32_t u = __shfl_xor_sync(0xffffffffu, v, o);
+                v = (lane & o) ? (v & ~m) | ((u >> o) & m) : (v & m) | ((u << o) & ~m);
+            }
+            so[cw * kOutWords + lane] = v;  // word cw of the lane's descriptor
+        }
+        bar_sync_id(5, kEvalThreads);
+        if (dead) continue;
+        const size_t row = static_cast<size_t>(prm.row0) + it.kp0;
+        if (n == kChunks) {
+            // whole rows: 4 threads per 64-byte descriptor, 16 per 256-byte expanded row
+            if (ct < 4 * it.nk) {
+                const int r = ct >> 2, q = ct & 3;
+                reinterpret_cast<uint4*>(out + row * kDescBytes)[ct] =
+                    make_uint4(so[(4 * q) * kOutWords + r], so[(4 * q + 1) * kOutWords + r],
+                               so[(4 * q + 2) * kOutWords + r], so[(4 * q + 3) * kOutWords + r]);
+            }
+            if (exp_out && ct < 16 * it.nk)
+                reinterpret_cast<uint4*>(exp_out + row * kExpRowBytes)[ct] =
+                    expand_word_e2m1(so[(ct & 15) * kOutWords + (ct >> 4)]);
+        } else {
+            // a part of the batch: descriptor bytes [ca, cb), expanded bytes [8 ca, 8 cb)
+            const uint8_t* sb = reinterpret_cast<const uint8_t*>(so);
+            for (int x = ct; x < n * it.nk; x += kEvalThreads) {
+                const int r = x / n, c = it.ca + x - r * n;
+                const uint32_t byte = sb[4 * ((c >> 2) * kOutWords + r) + (c & 3)];
+                out[(row + r) * kDescBytes + c] = static_cast<uint8_t>(byte);
+                if (exp_out)
+                    reinterpret_cast<uint32_t*>(exp_out + (row + r) * kExpRowBytes)[c] = expand_byte_e2m1(byte);
+            }
+        }
+    }
+    if (dead && lane == 0) atomicOr(flags, kFlagTimeout);
+    tc_fence_before();
+    bar_sync_id(5, kEvalThreads);
+    if (warp == kEvalWarp0) {
+        tc_fence_after();
+        tmem_dealloc(S.tmem, kTmemCols);
     }
 }
 
@@ -630,51 +788,169 @@ __global__ void __launch_bounds__(kThreads, 1) extract_lanes_kernel(
 
 // Host-side precomputation for the extraction kernel ------------------------------
 
-static TileGeom tile_geom(int reach) {
-    TileGeom t;
-    const int rx = (reach + 15) / 16 * 16;  // x margin rounded to the 16-byte TMA granule
-    t.tw = kCell + 2 * rx;
-    // an odd number of 16-byte granules per row: rows then start in 8 different bank
-    // groups (an even number gives 2 or 4), so the gathers along a rotated window
-    // row collide less
+int window_reach(double scale) {
+    // corner of the window: |a|, |e| <= 24, so |offset| <= 24 sqrt(2) scale, rounded
+    return static_cast<int>(std::floor(24.0 * std::sqrt(2.0) * scale + 0.5 + 1e-6));
+}
+
+// Tile box of a reach: the window's samples at any column of a 16-byte granule.  Rows of
+// an odd number of 16-byte granules start in 8 different bank groups (an even number
+// gives 2 or 4), so the gathers along a rotated window collide less.
+static TileClass tile_class(int reach) {
+    TileClass t;
+    t.reach = reach;
+    t.tw = (2 * reach + 1 + 15 + 15) / 16 * 16;
     if ((t.tw / 16) % 2 == 0) t.tw += 16;
-    t.th = kCell + 2 * reach;
-    t.mx = -rx;
-    t.my = -reach;
+    t.th = 2 * reach + 1;
     return t;
 }
 
-int extract_tile_pitch(int reach) { return tile_geom(reach).tw; }
-
-// Per triplet: the window word holding the first pixel of each patch's top row and
-// the pixel's byte in it (LaneTriplets layout).
-void build_triplet_offsets(const latch_triplet* trip, uint32_t* out /* 2 per triplet */) {
-    for (int t = 0; t < kBits; ++t) {
-        const uint8_t* c = &trip[t].ax;
-        uint32_t word[3], shift[3];
-        for (int p = 0; p < 3; ++p) {
-            const int x0 = c[2 * p] - kPatchR, y0 = c[2 * p + 1] - kPatchR;
-            word[p] = static_cast<uint32_t>(y0 * kRowWords + (x0 >> 2));
-            shift[p] = static_cast<uint32_t>(x0 & 3);
+// At most kClasses box sizes for the scale table: the scales sorted by reach are cut into
+// groups, each served by its largest box, so that the bytes over the table are fewest.
+static void tile_classes(const double* scales, int n, TileClass (&cls)[kClasses], int8_t (&cls_of)[LATCH_MAX_SCALES]) {
+    int order[LATCH_MAX_SCALES];
+    for (int i = 0; i < n; ++i) order[i] = i;
+    for (int i = 1; i < n; ++i)
+        for (int j = i; j > 0 && scales[order[j]] < scales[order[j - 1]]; --j) {
+            const int t = order[j];
+            order[j] = order[j - 1];
+            order[j - 1] = t;
         }
-        out[2 * t] = word[0] | (word[1] << 16);
-        out[2 * t + 1] = word[2] | (shift[0] << 16) | (shift[1] << 18) | (shift[2] << 20);
+    auto box = [&](int hi) { return tile_class(window_reach(scales[order[hi]])); };  // of sorted scale hi
+    int64_t best = -1;
+    int cut1 = n, cut2 = n;  // groups [0, cut1), [cut1, cut2), [cut2, n); empty ones allowed
+    for (int a = 1; a <= n; ++a)
+        for (int b = a; b <= n; ++b) {
+            int64_t bytes = 0;
+            const int ends[3] = {a, b, n};
+            for (int c = 0, from = 0; c < 3; from = ends[c], ++c)
+                if (ends[c] > from) {
+                    const TileClass t = box(ends[c] - 1);
+                    bytes += static_cast<int64_t>(t.tw) * t.th * (ends[c] - from);
+                }
+            if (best < 0 || bytes < best) {
+                best = bytes;
+                cut1 = a;
+                cut2 = b;
+            }
+        }
+    const int ends[3] = {cut1, cut2, n};
+    for (int c = 0, from = 0; c < 3; from = ends[c], ++c) {
+        cls[c] = box((ends[c] > from ? ends[c] : n) - 1);
+        for (int i = from; i < ends[c]; ++i) cls_of[order[i]] = static_cast<int8_t>(c);
     }
 }
 
-static CellGrid cell_grid(const latch_image* img) {
-    CellGrid g;
-    g.width = img->width;
-    g.height = img->height;
-    g.gx = (img->width + 2 * kMargin + kCell - 1) / kCell;
-    g.gy = (img->height + 2 * kMargin + kCell - 1) / kCell;
-    return g;
+// The kernel's offset table of every (scale, bin) from the (dx, dy) pairs of
+// build_offset_tables: four 16-bit tile offsets per window word, relative to the sample
+// at (-reach, -reach), in builder order (unit by unit, one word per lane).
+void build_tile_offsets(const double* scales, int nscales, const int8_t* offsets, uint16_t* out) {
+    TileClass cls[kClasses];
+    int8_t cls_of[LATCH_MAX_SCALES];
+    tile_classes(scales, nscales, cls, cls_of);
+    for (int t = 0; t < nscales * kBins; ++t) {
+        const TileClass& k = cls[cls_of[t / kBins]];
+        const int8_t* src = offsets + static_cast<size_t>(t) * kWinPix * 2;
+        uint16_t* dst = out + static_cast<size_t>(t) * kWinPix;
+        for (int blk = 0; blk < kBlocks; ++blk)
+            for (int l = 0; l < kBlockWords; ++l) {
+                const int cx = 4 * (blk % 3) + (l & 3), y = 8 * (blk / 3) + (l >> 2);
+                for (int q = 0; q < 4; ++q) {
+                    const int8_t* d = src + 2 * (y * kWin + 4 * cx + q);
+                    dst[(blk * kBlockWords + l) * 4 + q] =
+                        static_cast<uint16_t>((d[1] + k.reach) * k.tw + d[0] + k.reach);
+                }
+            }
+    }
 }
 
-// Two buffers of 32 windows, then two tiles (128 bytes of alignment slack).  At the
-// largest reach 221 KB (+5 KB static): one block per SM.
-static size_t extract_smem_bytes(const TileGeom& tg) {
-    return 128 + 2 * static_cast<size_t>(kBatch) * kLaneWords * 4 + 2 * ((static_cast<size_t>(tg.tw) * tg.th + 127) / 128 * 128);
+// Whether quarter Q holds the patch of size x size pixels at (x0, y0), and the three word
+// columns that a patch which does not start at a word is read from.
+static bool patch_in(const Quarter& Q, int x0, int y0, int size) {
+    const int x = x0 - Q.b0, y = y0 - Q.r0;
+    return x >= 0 && x + size <= 4 * Q.nc && y >= 0 && y + size <= Q.nr &&
+           ((x & 3) == 0 || ((x >> 2) + 2) * Q.nr + y <= kTmLast);
+}
+
+// The triplet table as the evaluators read it (LaneTriplets) for patches of `size` x
+// `size` pixels (7, or 8 when weighted): every triplet goes to the quarter in which it
+// costs least, with as many triplets in each as their fits allow.
+void plan_triplets(const latch_triplet* trip, int size, LaneTripletPlan* plan) {
+    // clocks of triplet t in quarter q (as measured): more with every patch that does not
+    // start at a word, and most with rows from shared memory; < 0: does not fit
+    constexpr int kCost = 72, kShiftCost = 9, kExtCost = 230;
+    int cost[kBits][kQuarters];
+    int8_t in[kBits];
+    int load[kQuarters] = {};
+    for (int t = 0; t < kBits; ++t) {
+        const uint8_t* c = &trip[t].ax;
+        for (int q = 0; q < kQuarters; ++q) {
+            const Quarter Q = quarter_of(q);
+            int shifts = 0;
+            bool all = true;
+            for (int p = 0; p < 3; ++p) {
+                const int x0 = c[2 * p] - kPatchR, y0 = c[2 * p + 1] - kPatchR;
+                all = all && patch_in(Q, x0, y0, size);
+                shifts += ((x0 - Q.b0) & 3) != 0;
+            }
+            cost[t][q] = all ? kCost + shifts * kShiftCost : q == 0 ? kCost + 3 * kShiftCost + kExtCost : -1;
+        }
+        in[t] = 0;
+        for (int q = 1; q < kQuarters; ++q)
+            if (cost[t][q] >= 0 && cost[t][q] < cost[t][in[t]]) in[t] = static_cast<int8_t>(q);
+        load[in[t]] += cost[t][in[t]];
+    }
+    // move triplets between quarters, each time the move that costs least among those out
+    // of the fullest quarter that has one (one that lowers the load of the two)
+    for (int moves = 0; moves < 4 * kBits; ++moves) {
+        int best = -1, to = 0, least = 0;
+        int below = INT32_MAX;
+        while (best < 0) {
+            int full = -1;
+            for (int q = 0; q < kQuarters; ++q)
+                if (load[q] < below && (full < 0 || load[q] > load[full])) full = q;
+            if (full < 0) break;
+            below = load[full];
+            for (int t = 0; t < kBits; ++t)
+                for (int q = 0; q < kQuarters; ++q) {
+                    if (in[t] != full || cost[t][q] < 0 || load[q] + cost[t][q] >= load[full]) continue;
+                    const int d = cost[t][q] - cost[t][full];
+                    if (best < 0 || d < least) {
+                        best = t;
+                        to = q;
+                        least = d;
+                    }
+                }
+        }
+        if (best < 0) break;
+        load[in[best]] -= cost[best][in[best]];
+        load[to] += cost[best][to];
+        in[best] = static_cast<int8_t>(to);
+    }
+    int at = 0;
+    for (int q = 0; q < kQuarters; ++q) {
+        const Quarter Q = quarter_of(q);
+        uint32_t word[3];
+        for (int cls = 0; cls < kTripClasses; ++cls) {
+            plan->start[q][cls] = static_cast<int16_t>(at);
+            for (int t = 0; t < kBits; ++t) {
+                if (in[t] != q) continue;
+                const uint8_t* c = &trip[t].ax;
+                int own = 0;
+                for (int p = 0; p < 3; ++p) {
+                    const int x0 = c[2 * p] - kPatchR - Q.b0, y0 = c[2 * p + 1] - kPatchR - Q.r0;
+                    word[p] = static_cast<uint32_t>(8 * (x0 & 3)) | static_cast<uint32_t>((x0 >> 2) * Q.nr + y0) << 16;
+                    own |= (x0 & 3) ? 1 << p : 0;
+                    if (!patch_in(Q, c[2 * p] - kPatchR, c[2 * p + 1] - kPatchR, size)) own |= 8;
+                }
+                if ((own & 8 ? 8 : own) != cls) continue;
+                word[0] |= static_cast<uint32_t>(t) << 5;
+                for (int p = 0; p < 3; ++p) plan->e[p][at] = word[p];
+                ++at;
+            }
+        }
+        plan->start[q][kTripClasses] = static_cast<int16_t>(at);
+    }
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -694,173 +970,110 @@ static EncodeTiledFn extract_encode_fn() {
     return fn;
 }
 
-// Scratch of one launch over images [i0, i1): sorted keypoint records, ranks, then
-// the region the host zeroes: counters, image totals, image arrival counters, cell
-// counts.
-struct ChunkLayout {
-    size_t recs, rank, zero, counters, img_tot, img_done, cells, total;
-    int64_t ncell, nkp;
-};
-
-static ChunkLayout chunk_layout(const latch_image* imgs, const int64_t* n, int i0, int i1) {
-    ChunkLayout l;
-    l.ncell = 0;
-    l.nkp = 0;
-    for (int i = i0; i < i1; ++i) {
-        const CellGrid g = cell_grid(&imgs[i]);
-        l.ncell += static_cast<int64_t>(g.gx) * g.gy;
-        l.nkp += n[i];
-    }
-    l.recs = 0;  // int4, 16-byte aligned
-    l.rank = l.recs + static_cast<size_t>(l.nkp) * sizeof(int4);
-    l.zero = (l.rank + static_cast<size_t>(l.nkp) * sizeof(int) + 255) / 256 * 256;
-    l.counters = l.zero;
-    l.img_tot = l.counters + 16;
-    l.img_done = l.img_tot + 64 * sizeof(int);
-    l.cells = l.img_done + 64 * sizeof(int);
-    l.total = (l.cells + static_cast<size_t>(l.ncell) * sizeof(int) + 255) / 256 * 256;
-    return l;
-}
-
 static constexpr int kBatchImages = 64;  // images per launch in the batched form
-
-size_t extract_batch_scratch_bytes(const latch_image* imgs, const int64_t* n, int count) {
-    size_t total = 0;
-    for (int i0 = 0; i0 < count; i0 += kBatchImages) {
-        const int i1 = i0 + kBatchImages < count ? i0 + kBatchImages : count;
-        total += chunk_layout(imgs, n, i0, i1).total;
-    }
-    return total;
-}
-
-size_t extract_scratch_bytes(const latch_image* img, int64_t n) { return extract_batch_scratch_bytes(img, &n, 1); }
+static_assert(sizeof(ExtractParams<kBatchImages>) + sizeof(LaneTriplets) + sizeof(PatchWeights) + 64 <= 32764,
+              "kernel parameter space");
 
 template <int NI, bool kWeighted>
 static cudaError_t set_extract_attributes() {
-    cudaError_t e = cudaFuncSetAttribute(extract_lanes_kernel<NI, kWeighted>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(extract_smem_bytes(tile_geom(kMaxReach + 1))));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(extract_lanes_kernel<NI, kWeighted>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 100);
-    return e;
+    return cudaFuncSetAttribute(extract_lanes_kernel<NI, kWeighted>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(kDynSmem));
 }
 
 template <int NI>
 static cudaError_t launch_chunk(const latch_context* ctx, const latch_image* imgs, const int64_t* kp0,
                                 const int64_t* n, int i0, int i1, const latch_keypoint* d_kps, uint8_t* d_out,
-                                uint8_t* exp_out, uint8_t* scratch, cudaStream_t stream,
-                                uint32_t* flags, const int32_t* n_dev) {
+                                uint8_t* exp_out, cudaStream_t stream, uint32_t* flags, const int32_t* n_dev) {
     static unsigned long long attr_done[2] = {0, 0};
-    const TileGeom tg = tile_geom(ctx->reach);
     cudaError_t e = ctx->weighted ? once_per_device(&attr_done[1], set_extract_attributes<NI, true>)
                                   : once_per_device(&attr_done[0], set_extract_attributes<NI, false>);
     if (e != cudaSuccess) return e;
     EncodeTiledFn enc = extract_encode_fn();
     if (!enc) return cudaErrorNotSupported;
-    const ChunkLayout l = chunk_layout(imgs, n, i0, i1);
-    int4* recs = reinterpret_cast<int4*>(scratch + l.recs);
-    int* rank = reinterpret_cast<int*>(scratch + l.rank);
-    int* counters = reinterpret_cast<int*>(scratch + l.counters);
-    int* img_tot = reinterpret_cast<int*>(scratch + l.img_tot);
-    int* img_done = reinterpret_cast<int*>(scratch + l.img_done);
-    int* cells = reinterpret_cast<int*>(scratch + l.cells);
-
-    ExtractParams<NI>* prm = new ExtractParams<NI>;
-    prm->count = i1 - i0;
-    prm->nscales = ctx->nscales;
-    prm->tg = tg;
-    prm->n_dev = n_dev;
-    int64_t cell0 = 0;
-    int blocks = 0;
+    struct Params {
+        ExtractParams<NI> prm;
+        LaneTriplets tt;
+        PatchWeights pw;
+    };
+    Params* p = new (std::nothrow) Params;
+    if (!p) return cudaErrorMemoryAllocation;
+    ExtractParams<NI>& prm = p->prm;
+    tile_classes(ctx->scales, ctx->nscales, prm.cls, prm.cls_of);
+    prm.count = i1 - i0;
+    prm.row0 = static_cast<int32_t>(kp0[i0]);
+    prm.nscales = ctx->nscales;
+    prm.min_batch = ctx->item_kps;
+    prm.n_dev = n_dev;
+    int64_t total = 0;
     for (int i = i0; i < i1; ++i) {
         const int j = i - i0;
-        const CellGrid g = cell_grid(&imgs[i]);
-        prm->grid[j] = g;
-        prm->kp0[j] = static_cast<int32_t>(kp0[i]);
-        prm->n[j] = static_cast<int32_t>(n[i]);
-        prm->cell0[j] = static_cast<int32_t>(cell0);
-        prm->blk0[j] = blocks;
-        cell0 += static_cast<int64_t>(g.gx) * g.gy;
-        blocks += static_cast<int>((n[i] + kSortKps - 1) / kSortKps);
+        prm.width[j] = imgs[i].width;
+        prm.height[j] = imgs[i].height;
+        prm.first[j] = static_cast<int32_t>(total);
+        total += n[i];
         cuuint64_t dims[2] = {static_cast<cuuint64_t>(imgs[i].width), static_cast<cuuint64_t>(imgs[i].height)};
         cuuint64_t strides[1] = {static_cast<cuuint64_t>(imgs[i].pitch)};
-        cuuint32_t box[2] = {static_cast<cuuint32_t>(tg.tw), static_cast<cuuint32_t>(tg.th)};
         cuuint32_t estr[2] = {1, 1};
-        if (enc(&prm->map[j], CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t*>(imgs[i].data), dims, strides, box,
-                estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
-            delete prm;
-            return cudaErrorInvalidValue;
+        for (int c = 0; c < kClasses; ++c) {
+            CUtensorMap* map = &prm.map[j * kClasses + c];
+            if (c > 0 && prm.cls[c].tw == prm.cls[c - 1].tw && prm.cls[c].th == prm.cls[c - 1].th) {
+                *map = map[-1];
+                continue;
+            }
+            cuuint32_t box[2] = {static_cast<cuuint32_t>(prm.cls[c].tw), static_cast<cuuint32_t>(prm.cls[c].th)};
+            if (enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t*>(imgs[i].data), dims, strides, box,
+                    estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                    CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
+                delete p;
+                return cudaErrorInvalidValue;
+            }
         }
     }
-    e = cudaMemsetAsync(scratch + l.zero, 0, l.total - l.zero, stream);
-    if (e == cudaSuccess)
-        e = launch_chained(sort_count_kernel<NI>, dim3(blocks), dim3(kSortThreads), 0, stream, *prm, d_kps, cells,
-                           rank, img_tot, img_done, reinterpret_cast<uint4*>(d_out),
-                           reinterpret_cast<uint4*>(exp_out), flags);
-    if (e == cudaSuccess)
-        e = launch_chained(sort_scatter_kernel<NI>, dim3(blocks), dim3(kSortThreads), 0, stream, *prm, d_kps,
-                           static_cast<const int*>(cells), static_cast<const int*>(rank),
-                           static_cast<const int*>(img_tot), counters, recs);
-    LaneTriplets* tt = e == cudaSuccess ? new LaneTriplets : nullptr;
-    if (tt) {
-        static_assert(sizeof(LaneTriplets) == sizeof(ctx->h_trip_offsets), "triplet table layout");
-        memcpy(tt, ctx->h_trip_offsets, sizeof(LaneTriplets));
-        // the chunks are split evenly over the blocks, at least item_kps keypoints' worth each
-        const int64_t want = (l.nkp + ctx->item_kps - 1) / ctx->item_kps;
-        const int64_t grid = want < ctx->sm_count ? want : ctx->sm_count;
-        PatchWeights pw;
-        for (int i = 0; i < 64; ++i) pw.w[i] = ctx->patch_weights[i];
-        e = launch_chained(ctx->weighted ? extract_lanes_kernel<NI, true> : extract_lanes_kernel<NI, false>,
-                           dim3(static_cast<unsigned>(grid)), dim3(kThreads), extract_smem_bytes(tg), stream, *prm, *tt,
-                           pw, static_cast<const int4*>(recs), static_cast<const int*>(counters), ctx->d_tile_offsets,
-                           d_out, exp_out, flags);
-        delete tt;
-    }
-    delete prm;
+    prm.n = static_cast<int32_t>(total);
+    static_assert(sizeof(LaneTriplets) == sizeof(ctx->trip_plan), "triplet table layout");
+    memcpy(&p->tt, &ctx->trip_plan, sizeof(LaneTriplets));
+    for (int i = 0; i < 64; ++i) p->pw.w[i] = ctx->patch_weights[i];
+    e = launch_chained(ctx->weighted ? extract_lanes_kernel<NI, true> : extract_lanes_kernel<NI, false>,
+                       dim3(static_cast<unsigned>(ctx->sm_count)), dim3(kThreads), kDynSmem, stream, prm, p->tt, p->pw,
+                       d_kps, reinterpret_cast<const uint2*>(ctx->d_tile_offsets), d_out, exp_out, flags);
+    delete p;
     return e;
 }
 
 cudaError_t launch_extract_batch(const latch_context* ctx, const latch_image* imgs, const int64_t* kp0,
                                  const int64_t* n, int count, const latch_keypoint* d_kps, uint8_t* d_out,
-                                 void* scratch, cudaStream_t stream, uint8_t* exp_out, uint32_t* flags) {
-    uint8_t* base = static_cast<uint8_t*>(scratch);
+                                 cudaStream_t stream, uint8_t* exp_out, uint32_t* flags) {
     if (!flags) flags = ctx->d_flags;
     for (int i0 = 0; i0 < count; i0 += kBatchImages) {
         const int i1 = i0 + kBatchImages < count ? i0 + kBatchImages : count;
         int64_t nk = 0;
         for (int i = i0; i < i1; ++i) nk += n[i];
-        if (nk > 0) {
-            // the kernel parameters hold one tensor map per image: the smallest
-            // instance that fits keeps the launch's parameter block small
-            const int ni = i1 - i0;
-            const cudaError_t e =
-                ni == 1    ? launch_chunk<1>(ctx, imgs, kp0, n, i0, i1, d_kps, d_out, exp_out, base, stream, flags, nullptr)
-                : ni <= 4  ? launch_chunk<4>(ctx, imgs, kp0, n, i0, i1, d_kps, d_out, exp_out, base, stream, flags, nullptr)
-                : ni <= 16 ? launch_chunk<16>(ctx, imgs, kp0, n, i0, i1, d_kps, d_out, exp_out, base, stream, flags, nullptr)
-                           : launch_chunk<kBatchImages>(ctx, imgs, kp0, n, i0, i1, d_kps, d_out, exp_out, base,
-                                                        stream, flags, nullptr);
-            if (e != cudaSuccess) return e;
-        }
-        base += chunk_layout(imgs, n, i0, i1).total;
+        if (nk == 0) continue;
+        // the kernel parameters hold the images' tensor maps: the smallest instance that
+        // fits keeps the launch's parameter block small
+        const int ni = i1 - i0;
+        const cudaError_t e =
+            ni == 1    ? launch_chunk<1>(ctx, imgs, kp0, n, i0, i1, d_kps, d_out, exp_out, stream, flags, nullptr)
+            : ni <= 4  ? launch_chunk<4>(ctx, imgs, kp0, n, i0, i1, d_kps, d_out, exp_out, stream, flags, nullptr)
+            : ni <= 16 ? launch_chunk<16>(ctx, imgs, kp0, n, i0, i1, d_kps, d_out, exp_out, stream, flags, nullptr)
+                       : launch_chunk<kBatchImages>(ctx, imgs, kp0, n, i0, i1, d_kps, d_out, exp_out, stream, flags,
+                                                    nullptr);
+        if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
 cudaError_t launch_extract(const latch_context* ctx, const latch_image* img, const latch_keypoint* d_kps, int32_t n,
-                           uint8_t* d_out, void* scratch, cudaStream_t stream) {
+                           uint8_t* d_out, cudaStream_t stream) {
     const int64_t kp0 = 0, nn = n;
-    return launch_extract_batch(ctx, img, &kp0, &nn, 1, d_kps, d_out, scratch, stream, nullptr);
+    return launch_extract_batch(ctx, img, &kp0, &nn, 1, d_kps, d_out, stream, nullptr);
 }
 
 cudaError_t launch_extract_dev_count(const latch_context* ctx, const latch_image* img, const latch_keypoint* d_kps,
-                                     int32_t max_n, const int32_t* d_n, uint8_t* d_out, void* scratch,
-                                     cudaStream_t stream) {
+                                     int32_t max_n, const int32_t* d_n, uint8_t* d_out, cudaStream_t stream) {
     if (max_n <= 0) return cudaSuccess;
     const int64_t kp0 = 0, nn = max_n;
-    return launch_chunk<1>(ctx, img, &kp0, &nn, 0, 1, d_kps, d_out, nullptr, static_cast<uint8_t*>(scratch),
-                           stream, ctx->d_flags, d_n);
+    return launch_chunk<1>(ctx, img, &kp0, &nn, 0, 1, d_kps, d_out, nullptr, stream, ctx->d_flags, d_n);
 }
 
 }  // namespace latch

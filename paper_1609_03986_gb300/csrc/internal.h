@@ -20,7 +20,6 @@ constexpr int kDescBytes = LATCH_DESC_BYTES;
 constexpr int kDescWords = kDescBytes / 4;  // 16
 constexpr int kBins = LATCH_ANGLE_BINS;
 constexpr double kMaxScale = 2.25;
-constexpr int kMaxReach = 77;               // max |offset| at scale 2.25 (24*sqrt(2)*2.25 = 76.4)
 
 // The tensor matcher's input row of one descriptor: its 512 bits as 4-bit E2M1
 // floats, two per byte, bit t -> value t = 1 - 2 bit (+1.0 = 0x2 when clear, -1.0 =
@@ -53,12 +52,16 @@ enum : uint32_t { kFlagBadScale = 1u, kFlagTimeout = 2u };
 // Host-built sample-offset tables (tables.cpp).  For each scale s and angle bin b,
 // kWinPix entries of (dx, dy) as int8 pairs, entry index v * 48 + u.
 void build_offset_tables(const double* scales, int nscales, int8_t* out /* nscales*32*2304*2 */);
-int max_reach(const double* scales, int nscales);
-// Staged-tile row pitch of the extraction kernel for a given reach.
-int extract_tile_pitch(int reach);
-// Window words and byte shifts of every triplet's three patches (the extraction
-// kernel's triplet parameter).
-void build_triplet_offsets(const latch_triplet* trip, uint32_t* out /* 2 per triplet */);
+// Largest |offset| of a window sample at this scale.
+int window_reach(double scale);
+// The extraction kernel's tile-offset tables (extract.cu) from those (dx, dy) tables.
+void build_tile_offsets(const double* scales, int nscales, const int8_t* offsets, uint16_t* out /* nscales*32*2304 */);
+// The extraction kernel's triplet parameter (extract.cu, LaneTriplets).
+struct LaneTripletPlan {
+    uint32_t e[3][LATCH_TRIPLETS];
+    int16_t start[4][10];
+};
+void plan_triplets(const latch_triplet* trip, int size, LaneTripletPlan* plan);
 
 struct Scratch {
     void* ptr = nullptr;
@@ -80,21 +83,20 @@ struct latch_context {
     int sm_count = 0;
     int nscales = 0;
     double scales[LATCH_MAX_SCALES] = {};
-    int reach = 0;                       // max |offset| over the scale table
-    int16_t* d_tile_offsets = nullptr;   // nscales * 32 * 2304 (+16 pad) tile offsets dy * pitch + dx
+    uint16_t* d_tile_offsets = nullptr;  // nscales * 32 * 2304 tile offsets (build_tile_offsets)
     latch_triplet h_trip[LATCH_TRIPLETS] = {};
     bool has_trip = false;
-    uint32_t h_trip_offsets[2 * LATCH_TRIPLETS] = {};
+    latch::LaneTripletPlan trip_plan = {};  // of h_trip and the patch size
     bool weighted = false;               // 8x8 weighted patches (latch_set_patch_weights) instead of 7x7
     int32_t patch_weights[64] = {};
     uint32_t* d_flags = nullptr;         // device error word
-    int32_t item_kps = 16;               // extraction: fewest keypoints per block (latch_autotune)
+    int32_t item_kps = 16;               // extraction: fewest keypoints per batch (latch_autotune)
     // tracing (latch_trace_enable): per batch run, events before extraction, between
     // extraction and matching, and after matching
     cudaEvent_t* trace_ev = nullptr;
     int32_t trace_cap = 0, trace_n = 0;
     int64_t tensor_min_pairs = int64_t(1) << 22;  // matching: AUTO uses the tensor path from here
-    latch::Scratch scratch[5];           // grow-only scratch regions (4: detection)
+    latch::Scratch scratch[4];           // grow-only: CUDA-core matching, tensor matching, batch, detection
     // latch_batch_run_host: two staging sets used alternately, upload stream
     latch::HostStaging staging[2];
     cudaStream_t up_stream = nullptr;
@@ -143,21 +145,19 @@ cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size
 
 // Kernel launchers (one per .cu file); return cudaGetLastError() of the launch.
 cudaError_t launch_extract(const latch_context* ctx, const latch_image* img, const latch_keypoint* d_kps, int32_t n,
-                           uint8_t* d_out, void* scratch, cudaStream_t stream);
-size_t extract_scratch_bytes(const latch_image* img, int64_t n);
-// Images [0, count) with keypoints d_kps[kp0[i] .. kp0[i] + n[i]) -> d_out rows at the same positions.
+                           uint8_t* d_out, cudaStream_t stream);
+// Images [0, count) with keypoints d_kps[kp0[i] .. kp0[i] + n[i]) -> d_out rows at the same positions
+// (kp0[i + 1] = kp0[i] + n[i]).
 // When exp_out is not NULL, row r of the tensor matcher's input (kExpRowBytes bytes, E2M1 +-1.0
 // per bit) is written as well.
 // `flags`: the device error word the kernels raise flags in (NULL: the context's).
 cudaError_t launch_extract_batch(const latch_context* ctx, const latch_image* imgs, const int64_t* kp0,
                                  const int64_t* n, int count, const latch_keypoint* d_kps, uint8_t* d_out,
-                                 void* scratch, cudaStream_t stream, uint8_t* exp_out, uint32_t* flags = nullptr);
-size_t extract_batch_scratch_bytes(const latch_image* imgs, const int64_t* n, int count);
+                                 cudaStream_t stream, uint8_t* exp_out, uint32_t* flags = nullptr);
 // One image whose keypoint count is on the device (*d_n, at most max_n keypoints in
-// d_kps); scratch as extract_scratch_bytes(img, max_n).
+// d_kps).
 cudaError_t launch_extract_dev_count(const latch_context* ctx, const latch_image* img, const latch_keypoint* d_kps,
-                                     int32_t max_n, const int32_t* d_n, uint8_t* d_out, void* scratch,
-                                     cudaStream_t stream);
+                                     int32_t max_n, const int32_t* d_n, uint8_t* d_out, cudaStream_t stream);
 
 // Oriented FAST keypoints (detect.cu) of the pyramid levels scales[0 .. nlev) (each >= 1;
 // scale 1 is the image itself), level l's keypoints given scale index scale_idx[l]:

@@ -116,13 +116,11 @@ latch_status sfail(latch_session* s, latch_status st, const char* msg) {
     return st;
 }
 
-// Device bytes one request needs in a lane (image, keypoints, descriptors, matches,
-// its share of the extraction scratch) -- the partial records of the match are
-// budgeted per batch.
+// Device bytes one request needs in a lane (image, keypoints, descriptors, matches) --
+// the partial records of the match are budgeted per batch.
 size_t request_bytes(const latch_request& r) {
-    const latch_image img{nullptr, r.width, r.height, dev_pitch(r.width)};
     return round_up(static_cast<size_t>(r.height) * dev_pitch(r.width), 256) +
-           round_up(static_cast<size_t>(r.n) * (12 + 64 + 16), 256) + extract_scratch_bytes(&img, r.n) + 1024;
+           round_up(static_cast<size_t>(r.n) * (12 + 64 + 16), 256) + 1024;
 }
 
 struct Carve {
@@ -166,8 +164,6 @@ latch_status run_batch(latch_session* s, int li, DoneArg* done) {
         if (e == cudaSuccess && r.n > 0)
             e = cudaMemcpyAsync(d_kps + kp0[i], r.h_kps, static_cast<size_t>(r.n) * 12, cudaMemcpyHostToDevice, st);
     }
-    const size_t ext_bytes = extract_batch_scratch_bytes(imgs.data(), n.data(), nb);
-    uint8_t* ext_scratch = cv.take(ext_bytes);
     // match problems: request i's query rows -> its gallery
     MatchBatch* mb = L.mb;
     for (int i = 0; i < nb; ++i) {
@@ -184,12 +180,12 @@ latch_status run_batch(latch_session* s, int li, DoneArg* done) {
     plan_match_batch(mb, nb, s->ctx->sm_count);
     uint64_t* partials = reinterpret_cast<uint64_t*>(cv.take(match_tc_partial_bytes(*mb) + 16));
     int32_t* tile_cnt = reinterpret_cast<int32_t*>(cv.take(match_tc_counter_bytes(mb->tiles)));
-    if (!ext_scratch || !partials || !tile_cnt) e = cudaErrorMemoryAllocation;  // admission bug guard
+    if (!partials || !tile_cnt) e = cudaErrorMemoryAllocation;  // admission bug guard
     if (e == cudaSuccess) e = cudaMemsetAsync(L.d_flags, 0, sizeof(uint32_t), st);
     if (e == cudaSuccess && total > 0) e = cudaMemsetAsync(tile_cnt, 0, match_tc_counter_bytes(mb->tiles), st);
     // the extraction writes the queries' expanded rows into the lane's arena rows
     if (e == cudaSuccess && total > 0)
-        e = launch_extract_batch(s->ctx, imgs.data(), kp0.data(), n.data(), nb, d_kps, d_desc, ext_scratch, st,
+        e = launch_extract_batch(s->ctx, imgs.data(), kp0.data(), n.data(), nb, d_kps, d_desc, st,
                                  s->arena + L.qrow0 * kExpRowBytes, L.d_flags);
     if (e == cudaSuccess && total > 0)
         e = launch_match_tc_rows(*mb, s->arena, s->arena_rows, partials, tile_cnt, d_match, L.d_flags, st);

@@ -61,11 +61,4 @@ void build_offset_tables(const double* scales, int nscales, int8_t* out) {
     }
 }
 
-int max_reach(const double* scales, int nscales) {
-    double m = 0.0;
-    for (int i = 0; i < nscales; ++i) m = scales[i] > m ? scales[i] : m;
-    // corner of the window: |a|, |e| <= 24, so |offset| <= 24*sqrt(2)*s, then rounding
-    return static_cast<int>(std::ceil(24.0 * std::sqrt(2.0) * m)) + 1;
-}
-
 }  // namespace latch
