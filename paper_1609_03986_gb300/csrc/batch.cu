@@ -69,7 +69,7 @@ latch_status plan_batch(latch_context* ctx, const latch_batch_desc* b, BatchPlan
     for (int p0 = 0; p0 < b->n_pairs; p0 += kMaxProblems) {
         const int p1 = p0 + kMaxProblems < b->n_pairs ? p0 + kMaxProblems : b->n_pairs;
         int64_t tiles = 0;
-        for (int p = p0; p < p1; ++p) tiles += (plan->n[b->h_pairs[2 * p]] + 127) / 128;
+        for (int p = p0; p < p1; ++p) tiles += match_tc_tiles(plan->n[b->h_pairs[2 * p]]);
         if (tiles > plan->max_tiles) plan->max_tiles = tiles;
     }
     for (int p0 = 0; p0 < b->n_pairs; p0 += kMaxProblems) {

@@ -65,7 +65,9 @@ __device__ __forceinline__ void top2_insert_u64(uint64_t key, uint64_t& k1, uint
     k2 = hi < k2 ? hi : k2;
 }
 
-void plan_match_batch(MatchBatch* b, int count, int64_t max_grid);
+// Query tiles of nq queries.
+int64_t match_tc_tiles(int64_t nq);
+void plan_match_batch(MatchBatch* b, int count, int64_t max_sms);
 // Scratch of the batched layout [expanded rows][arrival counters for
 // counter_tiles query tiles][partial records]; counter_tiles >= b.tiles.
 size_t match_tc_batch_scratch_bytes(int64_t rows, const MatchBatch& b, int64_t counter_tiles);
@@ -81,7 +83,7 @@ size_t match_tc_partial_bound(int64_t queries, int64_t problems, int64_t sms);
 cudaError_t launch_match_tc_batch(const MatchBatch& b, int64_t rows, int64_t counter_tiles, void* scratch,
                                   latch_match* out, uint32_t* flags, cudaStream_t stream);
 // Same with explicit buffers: `exp` holds `rows` expanded rows, `partials`
-// match_tc_partial_bytes(b) of scratch, `tile_cnt` b.tiles zero counters (NULL:
+// match_tc_partial_bytes(b) of scratch, `tile_cnt` match_tc_counter_bytes(b.tiles) of zero counters (NULL:
 // combine the records in a separate pass).
 cudaError_t launch_match_tc_rows(const MatchBatch& b, const uint8_t* exp, int64_t rows, uint64_t* partials,
                                  int32_t* tile_cnt, latch_match* out, uint32_t* flags, cudaStream_t stream);

@@ -10,37 +10,54 @@
 //
 // One launch serves a batch of matching problems (query set x train set pairs; a
 // single hamming_match call is a batch of one).  All descriptors live in one
-// expanded buffer (two TMA tensor maps over it: 128-row query boxes, 240-row train
-// boxes).  The units (problem, 128-query tile, 240-train tile) of all problems are
-// linearised and split into one contiguous range per block (one block per SM,
-// persistent):
-//   warp 0     TMA producer: the query tile (128 rows x 256 B, 32 KB) stays resident
-//              while consecutive units share it; train chunks (240 rows x 128 B, half
-//              of K) go through a 6-stage ring, 128-byte swizzle;
-//   warps 1-2  MMA issuers (even / odd units): per unit 8 tcgen05.mma (M=128,
-//              N=240, K=64) into one of two TMEM accumulators (columns 0 and 256; the
-//              constant scale factors in 496-511); warp 2 also allocates TMEM;
+// expanded buffer (two TMA tensor maps over it: 128-row query boxes, 120-row train
+// boxes).  The blocks work in pairs (clusters of two on the two SMs of a TPC, one block
+// per SM, persistent); a pair's MMAs (cta_group::2, M = 256) take a tile of 256 queries,
+// 128 in each block, and 240 train rows, 120 in each block's shared memory.  The units
+// (problem, 256-query tile, 240-train tile) of all problems are linearised and split into
+// one contiguous range per pair:
+//   warp 0     TMA producer of its block's half: the query rows (128 rows x 256 B, 32 KB)
+//              stay resident while consecutive units share them; train chunks (120 rows x
+//              128 B, half of K) go through a 12-stage ring, 128-byte swizzle; both
+//              blocks' copies complete on the first block's barriers;
+//   warps 1-2  MMA issuers, in the pair's first block (even / odd units): per unit 6
+//              tcgen05.mma (per 128-byte chunk of K = 256 values: K = 96, 96, 64) into one
+//              of two TMEM accumulators (columns 0 and 256 of both blocks; the constant
+//              scale factors in 496-511); their commits reach both blocks' barriers;
+//              warp 2 also allocates TMEM;
 //   warp 3     idle;
-//   warps 4-23 epilogue (one query row and 48 columns per thread): three reducing
-//              TMEM loads (tcgen05.ld.red .max) bring the 48 values and the largest
-//              of each 16, and the accumulator is released at once.  A group of 16
-//              whose largest value is below the row's bound costs nothing more: the
-//              bound is the smallest second-best distance any of the row's five
-//              column groups holds (shared memory), and a column displaces one of its
-//              own group's keys only with a larger value (later columns have larger
-//              train indices).  The others take the top-two update (a tournament over
-//              64 v - column, unique values that break ties to the lower index).  When
-//              the block leaves a query tile the row's two (distance << 32 | index)
-//              keys go to a partial record.  In a launch of at most
-//              kFusedUnitsPerBlock units per block the last block to leave a tile (a
-//              per-tile arrival counter) combines the records of its rows and writes
-//              their matches (ties to the lowest train index, ratio test).
-// The unit width is a compile-time choice (LATCH_TC_COLS): 160 gives three
-// accumulators in rotation (columns 0, 160, 320) and 32 columns per epilogue thread.
+//   warps 4-23 epilogue of the block's 128 rows (one query row and 48 columns per
+//              thread): three reducing TMEM loads (tcgen05.ld.red .max) bring the 48
+//              values and the largest of each 16, and the accumulator is released at
+//              once.  A group of 16 whose largest value is below the row's bound costs
+//              nothing more: the bound is the smallest second-best distance any of the
+//              row's five column groups holds (shared memory), and a column displaces one
+//              of its own group's keys only with a larger value (later columns have
+//              larger train indices).  The others take the top-two update (a tournament
+//              over 64 v - column, unique values that break ties to the lower index).
+//              When the pair leaves a query tile the row's two (distance << 32 | index)
+//              keys go to a partial record.  In a launch of at most kFusedUnitsPerPair
+//              units per pair the last block to leave a tile's half (an arrival counter
+//              each) combines the records of its rows and writes their matches (ties to
+//              the lowest train index, ratio test).
 // match_merge_kernel does the same combination as a separate pass; it serves longer
 // launches and the batches in which some problem has queries but an empty train set
 // (no unit, so no block visits its tiles).  All mbarrier waits are bounded (sm103.h); on a timeout
-// the block raises the device flag, drains its copies and MMAs, frees TMEM.
+// the block raises the device flag, lets its copies and MMAs end, frees TMEM.
+//
+// Why pairs and K = 96: shared memory (128 bytes per clock per SM) bounds the MMAs.  One
+// block alone (M = 128, N = 240) reads 94 KB of operands per unit and the copies write
+// 61 KB, 1,215 clocks (the kernel took 1,206 per unit; its MMAs at K = 64 need 960, and at
+// K = 96 they are no faster than 846 because of the operand reads).  In a pair each block
+// reads its own query rows but only half of the train rows, and copies half: 94 KB, 735
+// clocks, next to 720 of MMAs (K = 96 issues 1.5 times the products of K = 64 per clock).
+// Measured (GB300, before: single blocks, K = 64, an MMA thread of its own): 16,384 x
+// 1,048,576 descriptors 2,386 -> 1,783 us (943 clocks per unit), 10,000 x 10,000 46.3 ->
+// 43.4 us, a batch of 64 images and 476 pairs (3.4e11 distances) 59.8 -> 52.4 ms.  What is
+// left above 720 clocks is the accumulators' round trip (MMA end, commit, TMEM loads of 20
+// warps, arrivals of both blocks, next MMA: about 1,200 clocks for two accumulators in
+// flight); three accumulators of 160 columns are slower (2,357 us: the epilogue's time per
+// unit hardly depends on its columns).
 #include <cuda.h>
 
 #include <cmath>
@@ -55,22 +72,19 @@ namespace {
 
 using namespace sm103;
 
-constexpr int kRowsA = 128;             // rows per MMA (M) = queries per tile
-constexpr int kRowsQ = kRowsA;
-#ifndef LATCH_TC_COLS
-#define LATCH_TC_COLS 240
-#endif
-constexpr int kColsB = LATCH_TC_COLS;   // train rows per unit (N): 240 (two accumulators) or 160 (three)
+constexpr int kRowsA = 128;             // query rows per block
+constexpr int kRowsQ = 2 * kRowsA;      // query rows per tile (M of the pair's MMA)
+constexpr int kColsB = 240;             // train rows per unit (N)
+constexpr int kRowsB = kColsB / 2;      // of these in each block's shared memory
 constexpr int kRowsP = kRowsQ;          // partial records per tile slot: one per query row
 constexpr int kKBytes = kExpRowBytes;   // expanded descriptor: 512 x 4-bit
 constexpr int kChunk = 128;             // K bytes per swizzle atom / TMA box
 constexpr int kChunks = kKBytes / kChunk;
-constexpr int kMmaKBytes = 32;          // K bytes per MMA: 64 E2M1 values
-constexpr int kStages = kColsB > 192 ? 6 : 8;  // train chunks in flight (three / four units)
+constexpr int kStages = 12;             // train chunks in flight (six units)
 constexpr int kTileBytes = kRowsA * kChunk;   // 16 KB: a query chunk of 128 rows x 128 B (one TMA box)
-constexpr int kStageBytes = kColsB * kChunk;  // a train chunk of kColsB rows x 128 B (one TMA box)
-constexpr int kAccs = kColsB > 160 ? 2 : 3;    // TMEM accumulators in rotation (unit i uses i % kAccs)
-constexpr int kAccStride = kColsB > 160 ? 256 : kColsB;  // accumulator a at TMEM columns [a kAccStride, +kColsB)
+constexpr int kStageBytes = kRowsB * kChunk;  // 15 KB: a train chunk of 120 rows x 128 B (one TMA box)
+constexpr int kAccs = 2;                // TMEM accumulators in rotation (unit i uses i % kAccs)
+constexpr int kAccStride = 256;          // accumulator a at TMEM columns [a kAccStride, +kColsB)
 constexpr int kEpiWarps = 20;           // epilogue: 4 lane quarters x 5 column groups
 constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kThreads = 128 + kEpiThreads;         // producer, two MMA issuers, an idle warp, then the epilogue
@@ -81,11 +95,13 @@ constexpr int kLds = kColsPerThread / kLdCols;       // loads per unit and threa
 constexpr int kTmemCols = 512;
 constexpr uint32_t kSfaCol = (kAccs - 1) * kAccStride + kColsB;  // scale factors of A: 4 columns (128 rows)
 constexpr uint32_t kSfbCol = kSfaCol + 8;  // scale factors of B: 4 columns per 128 rows
-constexpr uint32_t kScaleOne = 0x7F7F7F7Fu;  // four UE8M0 scale factors 2^0 (columns 480-511 all hold it)
-constexpr uint32_t kIdesc = idesc_mxf4_e2m1(kRowsA, kColsB);
+constexpr uint32_t kScaleOne = 0x7F7F7F7Fu;  // four UE8M0 scale factors 2^0 (columns 496-511 all hold it)
+constexpr uint32_t kIdesc64 = idesc_mxf4_e2m1(kRowsQ, kColsB);
+constexpr uint32_t kIdesc96 = kIdesc64 | kIdescK96;
 constexpr int32_t kNoBound = 1024;      // a distance bound above every distance (512 bits)
-constexpr int64_t kFusedUnitsPerBlock = 64;  // longer launches combine the tiles' records in a separate pass
-constexpr int64_t kWholeTilesPerBlock = 8;   // batches with this many query tiles per block share whole tiles
+constexpr int64_t kFusedUnitsPerPair = 64;  // longer launches combine the tiles' records in a separate pass
+constexpr int64_t kWholeTilesPerPair = 8;   // batches with this many query tiles per pair share whole tiles
+static_assert(kStageBytes % 1024 == 0 && kTileBytes % 1024 == 0, "128-byte swizzle atoms");
 static_assert(kSfaCol % 8 == 0 && kSfbCol + 4 * ((kColsB + 127) / 128) <= kTmemCols, "TMEM columns overlap");
 static_assert(kColsPerThread == kLds * kLdCols && kColsB == kColGroups * kColsPerThread, "epilogue column split");
 static_assert(kColsB % 16 == 0 && kColsB <= 256 && kColsPerThread < 64 && kAccStride % 32 == 0, "unit shape");
@@ -97,16 +113,21 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
     return d;
 }
 
+// mbar_wait by a whole warp, which goes on together.
+__device__ __forceinline__ bool wait_all(uint64_t* bar, uint32_t parity, volatile int* abort) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort));
+}
+
 // Barrier of the epilogue threads (named barrier 1).
 __device__ __forceinline__ void group_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 
 struct Smem {
     // offsets in the 1024-aligned dynamic buffer
     static constexpr int a = 0;                                        // [kChunks] boxes of 16 KB
-    static constexpr int b = a + kChunks * kTileBytes;                 // [kStages] chunks of 20 KB
+    static constexpr int b = a + kChunks * kTileBytes;                 // [kStages] chunks of 15 KB
     static constexpr int part = b + kStages * kStageBytes;             // uint64 [kEpiThreads][2]
-    static constexpr int bound = part + kEpiThreads * 16;              // int32 [kRowsQ]
-    static constexpr int bars = bound + kRowsQ * 4;                    // uint64 barriers
+    static constexpr int bound = part + kEpiThreads * 16;              // int32 [kRowsA]
+    static constexpr int bars = bound + kRowsA * 4;                    // uint64 barriers
     static constexpr int nbars = 2 * kStages + 2 + 2 * kAccs + 2;
     static constexpr int misc = bars + nbars * 8;                      // tmem base, abort flag, last-arrival flag
     static constexpr int total = misc + 16;
@@ -114,7 +135,7 @@ struct Smem {
 constexpr int kSmemBytes = Smem::total + 1024;
 static_assert(kSmemBytes <= 227 * 1024, "shared memory per block");
 
-// Walks the units of block c: for every problem in turn, the block's share of that
+// Walks the units of pair c: for every problem in turn, the pair's share of that
 // problem's U units, [start(c'), start(c' + 1)) with start(x) = floor(x U / G) and
 // c' = (c - unit0) mod G (the rotation continues each problem where the previous
 // one ended, so problems smaller than G still spread over all blocks), without
@@ -314,7 +335,7 @@ __device__ __forceinline__ latch_match final_match(uint64_t k1, uint64_t k2, int
 // tile_cnt: per-query-tile arrival counters, zero at launch and zero again after a
 // complete launch; NULL = leave the combination to match_merge_kernel.
 template <int NP>
-__global__ void __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_constant__ CUtensorMap tmq,
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_constant__ CUtensorMap tmq,
                                                               const __grid_constant__ CUtensorMap tmt,
                                                               const __grid_constant__ MatchBatchT<NP> batch,
                                                               uint64_t* __restrict__ partials,
@@ -341,7 +362,8 @@ __global__ void __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_cons
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const int64_t c = blockIdx.x;
+    const int rank = static_cast<int>(blockIdx.x & 1);  // in the pair; rank 0's block issues the MMAs
+    const int64_t c = blockIdx.x >> 1;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; ++i) {
@@ -352,7 +374,7 @@ __global__ void __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_cons
         mbar_init(a_empty, 2);  // both MMA warps commit once per query tile
         for (int i = 0; i < kAccs; ++i) {
             mbar_init(&acc_full[i], 1);
-            mbar_init(&acc_empty[i], kEpiThreads / 32);
+            mbar_init(&acc_empty[i], 2 * kEpiWarps);  // both blocks' epilogue warps (rank 0's barrier)
         }
         mbar_init(&mma_done[0], 1);
         mbar_init(&mma_done[1], 1);
@@ -364,10 +386,10 @@ __global__ void __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_cons
         prefetch_tmap(&tmt);
     }
     if (warp == 2) {
-        tmem_alloc(tmem_slot, kTmemCols);
+        tmem_alloc_pair(tmem_slot, kTmemCols);
         tc_fence_before();
     }
-    for (int r = threadIdx.x; r < kRowsQ; r += kThreads) sBound[r] = kNoBound;
+    for (int r = threadIdx.x; r < kRowsA; r += kThreads) sBound[r] = kNoBound;
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
@@ -381,8 +403,9 @@ __global__ void __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_cons
     }
     tc_fence_before();
     __syncthreads();
+    cluster_sync();  // both blocks' barriers and scale factors are there
     tc_fence_after();
-    // everything above touched only this block's shared memory and TMEM
+    // everything above touched only this pair's shared memory and TMEM
     griddep_wait();
     griddep_launch_dependents();
 
@@ -393,9 +416,7 @@ __global__ void __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_cons
             it.init(batch, c);
             int stage = 0;
             uint32_t ring = 0, a_par = 0;
-            // bit s: stage s has a copy issued / the parity of its latest fill (bit masks
-            // rather than arrays, which a run-time index would put in local memory)
-            uint32_t filled = 0, fill_par = 0;
+            const uint32_t a_full0 = cluster_addr(smem_u32(a_full), 0), full0 = cluster_addr(smem_u32(full), 0);
             int64_t prev_g = -1;
             for (; !it.done(batch); it.next(batch, c)) {
                 const MatchProblem& P = batch.p[it.p];
@@ -406,10 +427,10 @@ __global__ void __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_cons
                         if (!mbar_wait(a_empty, a_par, abort)) break;
                         a_par ^= 1;
                     }
-                    mbar_arrive_expect_tx(a_full, kChunks * kTileBytes);
+                    if (rank == 0) mbar_arrive_expect_tx(a_full, 2 * kChunks * kTileBytes);
                     for (int kc = 0; kc < kChunks; ++kc)
-                        tma_load_2d(sA + kc * kTileBytes, &tmq, kc * kChunk, static_cast<int32_t>(P.q_row0 + m * kRowsQ),
-                                    a_full);
+                        tma_load_2d_pair(sA + kc * kTileBytes, &tmq, kc * kChunk,
+                                         static_cast<int32_t>(P.q_row0 + m * kRowsQ + rank * kRowsA), a_full0);
                     prev_g = g;
                 }
                 bool ok = true;
@@ -418,11 +439,10 @@ __global__ void __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_cons
                         ok = false;
                         break;
                     }
-                    mbar_arrive_expect_tx(&full[stage], kStageBytes);
-                    tma_load_2d(sB + stage * kStageBytes, &tmt, kc * kChunk, static_cast<int32_t>(it.t_row0 + n * kColsB),
-                                &full[stage]);
-                    filled |= 1u << stage;
-                    fill_par = (fill_par & ~(1u << stage)) | (ring << stage);
+                    if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * kStageBytes);
+                    tma_load_2d_pair(sB + stage * kStageBytes, &tmt, kc * kChunk,
+                                     static_cast<int32_t>(it.t_row0 + n * kColsB + rank * kRowsB),
+                                     full0 + 8u * static_cast<uint32_t>(stage));
                     if (++stage == kStages) {
                         stage = 0;
                         ring ^= 1;
@@ -431,26 +451,27 @@ __global__ void __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_cons
                 if (!ok) break;
             }
             if (*abort) {
-                // let copies still in flight land before the block exits (bounded)
+                // let copies still in flight land before the block exits (their barriers are in
+                // the other block, which may have given up: a fixed time)
                 const uint64_t t0 = globaltimer();
-                for (int s = 0; s < kStages; ++s)
-                    while (((filled >> s) & 1u) && !mbar_try_wait(&full[s], (fill_par >> s) & 1u) &&
-                           globaltimer() - t0 < 200000000ull) {
-                    }
-                if (prev_g >= 0)  // the last A load completes the a_full phase of parity a_par
-                    while (!mbar_try_wait(a_full, a_par) && globaltimer() - t0 < 200000000ull) {
-                    }
+                while (globaltimer() - t0 < 50000000ull) {
+                }
             }
         }
     } else if (warp == 1 || warp == 2) {
         // ---------------- MMA issuers: warp 1 issues the even units, warp 2 the odd ones
         // (a thread's tcgen05.mma waits until the tensor pipe takes it, so a single
         // issuer leaves the pipe idle while it waits on barriers between units; with two,
-        // one issuer's waits overlap the other's MMAs).  Unit i uses accumulator i % 3
+        // one issuer's waits overlap the other's MMAs).  Unit i uses accumulator i % 2
         // and stages 2 i, 2 i + 1 of the ring; both issuers walk every unit, wait for
         // every query tile and commit a_empty (count 2) at every tile's end. ----------------
-        if (lane == 0) {
+        if (rank == 0) {
+            // The whole warp walks the units and one elected lane issues: the loop's
+            // counters are uniform (shuffles tell the compiler so), so the descriptors live in
+            // uniform registers, as the MMA instruction takes them.  Issued from a branch of a
+            // single lane with per-thread counters, every MMA took about 60 clocks more.
             const int mine = warp - 1;
+            const bool issuer = elect_one();
             RunIter run;
             run.init(batch, c);
             uint32_t a_par = 0;
@@ -459,61 +480,69 @@ __global__ void __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_cons
             // adds a constant to them
             const uint64_t a_desc0 = umma_desc_sw128(smem_u32(sA));
             const uint64_t b_desc0 = umma_desc_sw128(smem_u32(sB));
-            const uint32_t sfa = tmem + kSfaCol, sfb = tmem + kSfbCol;
+            const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+            const uint32_t sfa = tm + kSfaCol, sfb = tm + kSfbCol;
             int i = 0;  // the run's first unit in the block's walk
             bool ok = true;
             for (; ok && !run.done(batch); run.next(batch, c)) {
-                if (!mbar_wait(a_full, a_par, abort)) break;  // every run is a new query tile
+                if (!wait_all(a_full, a_par, abort)) break;  // every run is a new query tile
                 a_par ^= 1;
-                const int end = i + run.len;
+                const int end = __shfl_sync(0xffffffffu, i + run.len, 0);
                 for (int j = i + ((i & 1) ^ mine); ok && j < end; j += 2) {
+                    // unit j reads ring positions 2 j and 2 j + 1; its first MMA overwrites D.  The
+                    // accumulator comes last: it is what the unit usually waits for, and the
+                    // MMAs can follow at once
                     const int acc = j % kAccs;
-                    if (!mbar_wait(&acc_empty[acc], static_cast<uint32_t>((j / kAccs) & 1) ^ 1u, abort)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t d = tmem + static_cast<uint32_t>(acc * kAccStride);
-                    // unit j reads ring positions 2 j and 2 j + 1; its first MMA overwrites D
 #pragma unroll
                     for (int kc = 0; kc < kChunks; ++kc) {
                         const int pos = kChunks * j + kc;
-                        const int stage = pos % kStages;
-                        if (!mbar_wait(&full[stage], static_cast<uint32_t>(pos / kStages) & 1u, abort)) {
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
+                        ok = ok && wait_all(&full[pos % kStages], static_cast<uint32_t>(pos / kStages) & 1u, abort);
+                    }
+                    ok = ok && wait_all(&acc_empty[acc], static_cast<uint32_t>((j / kAccs) & 1) ^ 1u, abort);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t d = tm + static_cast<uint32_t>(acc * kAccStride);
+#pragma unroll
+                    for (int kc = 0; kc < kChunks; ++kc) {
+                        const int stage = (kChunks * j + kc) % kStages;
                         const uint64_t bd = b_desc0 + static_cast<uint64_t>((stage * kStageBytes) >> 4);
                         const uint64_t ad = a_desc0 + static_cast<uint64_t>((kc * kTileBytes) >> 4);
-#pragma unroll
-                        for (int ks = 0; ks < kChunk / kMmaKBytes; ++ks)
-                            mma_mxf4(d, ad + static_cast<uint64_t>((ks * kMmaKBytes) >> 4),
-                                     bd + static_cast<uint64_t>((ks * kMmaKBytes) >> 4), kIdesc, sfa, sfb,
-                                     (kc | ks) != 0);
-                        mma_commit(&empty[stage]);
+                        // 256 values: K = 96, 96, 64 (48, 48 and 32 bytes: none crosses the swizzle atom)
+                        if (issuer) {
+                            mma_mxf4_pair(d, ad, bd, kIdesc96, sfa, sfb, kc != 0);
+                            mma_mxf4_pair(d, ad + 3, bd + 3, kIdesc96, sfa, sfb, 1);
+                            mma_mxf4_pair(d, ad + 6, bd + 6, kIdesc64, sfa, sfb, 1);
+                            mma_commit_pair(&empty[stage]);
+                            if (kc == kChunks - 1) mma_commit_pair(&acc_full[acc]);
+                        }
+                        __syncwarp();
                     }
-                    if (ok) mma_commit(&acc_full[acc]);
                 }
                 i = end;
-                if (ok) mma_commit(a_empty);
+                if (ok && issuer) mma_commit_pair(a_empty);
+                __syncwarp();
             }
             // every issued MMA has finished before TMEM is released
-            mma_commit(&mma_done[mine]);
-            const uint64_t t0 = globaltimer();
-            while (!mbar_try_wait(&mma_done[mine], 0) && globaltimer() - t0 < 200000000ull) {
+            if (issuer) {
+                mma_commit_pair(&mma_done[mine]);
+                const uint64_t t0 = globaltimer();
+                while (!mbar_try_wait(&mma_done[mine], 0) && globaltimer() - t0 < 200000000ull) {
+                }
             }
+            __syncwarp();
         }
     } else if (warp >= 4) {
         // ---------------- epilogue: kEpiWarps warps; thread = one query row x one
         // group of kColsPerThread accumulator columns.  The walk goes by runs (the
         // consecutive units of one query tile), so the per-unit path touches only
         // counters in registers; the problem table is read where a run ends. ----------------
-        const int et = threadIdx.x - 128;  // 0 .. kEpiThreads-1 = cg * kRowsQ + row_in_tile
+        const int et = threadIdx.x - 128;  // 0 .. kEpiThreads-1 = cg * kRowsA + row_in_block
         const int quarter = warp & 3;      // TMEM lane quarter this warp may access
         const int cg = (warp - 4) >> 2;    // column group [cg * kColsPerThread, +kColsPerThread)
         const int col0 = cg * kColsPerThread;
-        const int row_in_tile = quarter * 32 + lane;
+        const int row_in_block = quarter * 32 + lane;
+        const int row_in_tile = rank * kRowsA + row_in_block;
+        const uint32_t acc_empty0 = cluster_addr(smem_u32(acc_empty), 0);
         const uint32_t lane_base = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(col0);
         const float kNegInf = __int_as_float(0xff800000);
         RunIter run;
@@ -576,7 +605,7 @@ __global__ void __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_cons
                 if (k2 != kNoKey) {
                     const int32_t d2 = static_cast<int32_t>(k2 >> 32);
                     vown2 = static_cast<float>(514 - 2 * d2);
-                    atomicMin(&sBound[row_in_tile], d2);
+                    atomicMin(&sBound[row_in_block], d2);
                 }
             };
             const int32_t n_end = u.n + run.len;
@@ -601,11 +630,11 @@ __global__ void __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_cons
                     // (equal: when its index is lower than a key's of another group), i.e.
                     // with a value >= 512 - 2 bound, and only above the thread's second best
                     const float vmin = fmaxf(
-                        static_cast<float>(512 - 2 * *static_cast<volatile int32_t*>(&sBound[row_in_tile])), vown2);
+                        static_cast<float>(512 - 2 * *static_cast<volatile int32_t*>(&sBound[row_in_block])), vown2);
                     tmem_ld_wait();
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(&acc_empty[acc]);
+                    if (lane == 0) mbar_arrive_cluster(acc_empty0 + 8u * static_cast<uint32_t>(acc));
                     float e[kColsPerThread];
 #pragma unroll
                     for (int h = 0; h < kLds; ++h)
@@ -622,10 +651,14 @@ __global__ void __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_cons
                             }
                         }
                     }
-                    // only a group of 16 that reaches the row's bound takes the top-two update
+                    // only a group of 16 that reaches the row's bound takes the top-two update; one
+                    // vote sends the warp on when none does, which is the usual case
+                    static_assert(kLds == 3, "the vote below");
+                    if (__any_sync(0xffffffffu, fmax3(mx[0], mx[1], mx[2]) >= vmin)) {
 #pragma unroll
-                    for (int h = 0; h < kLds; ++h)
-                        if (__any_sync(0xffffffffu, mx[h] >= vmin)) update(e, h, n, vmin);
+                        for (int h = 0; h < kLds; ++h)
+                            if (__any_sync(0xffffffffu, mx[h] >= vmin)) update(e, h, n, vmin);
+                    }
                 }
                 if (++acc == kAccs) acc = 0;
             }
@@ -639,11 +672,11 @@ __global__ void __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_cons
             sPart[2 * et + 1] = k2;
             group_sync();  // every thread is past the run's last bound read
             if (cg == 0) {
-                sBound[row_in_tile] = kNoBound;
+                sBound[row_in_block] = kNoBound;
 #pragma unroll
                 for (int q = 1; q < kColGroups; ++q) {
-                    top2_insert_u64(sPart[2 * (q * kRowsQ + row_in_tile)], k1, k2);
-                    top2_insert_u64(sPart[2 * (q * kRowsQ + row_in_tile) + 1], k1, k2);
+                    top2_insert_u64(sPart[2 * (q * kRowsA + row_in_block)], k1, k2);
+                    top2_insert_u64(sPart[2 * (q * kRowsA + row_in_block) + 1], k1, k2);
                 }
                 if (batch.whole_tiles) {
                     // the block owns the whole tile: the row's two keys are final
@@ -658,10 +691,11 @@ __global__ void __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_cons
             }
             group_sync();  // the shared records are free for the next run
             if (tile_cnt && !batch.whole_tiles) {
-                // the last owner of the tile to arrive combines the records
+                // the last owner of the tile's half to arrive combines its records
                 if (et == 0) {
-                    const bool last = atomicAdd(&tile_cnt[g], 1) == tile_owner_count(batch, P, m) - 1;
-                    if (last) tile_cnt[g] = 0;  // no other block touches it again: leave it zero
+                    int32_t* cnt = &tile_cnt[2 * g + rank];
+                    const bool last = atomicAdd(cnt, 1) == tile_owner_count(batch, P, m) - 1;
+                    if (last) *cnt = 0;  // no other block touches it again: leave it zero
                     *last_arrival = last;
                 }
                 group_sync();
@@ -675,11 +709,13 @@ __global__ void __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_cons
             }
         }
     }
+    tc_fence_before();
     __syncthreads();
     if (threadIdx.x == 0 && *abort) atomicOr(flags, kFlagTimeout);
+    cluster_sync();  // the other block's MMAs, copies and arrivals are over too
     if (warp == 2) {
         tc_fence_after();
-        tmem_dealloc(tmem, kTmemCols);
+        tmem_dealloc_pair(tmem, kTmemCols);
     }
 }
 
@@ -712,6 +748,23 @@ __global__ void expand_kernel(const uint32_t* __restrict__ in, int64_t nwords, u
     griddep_launch_dependents();
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i < nwords) out[i] = expand_word_e2m1(in[i]);
+}
+
+// The same for a single problem: the query set, then the train set behind it, and the
+// matcher's arrival counters cleared, in one launch.  (Two expansions and a memset in
+// front of the matcher cost about 2 us more: 10,000 x 10,000 descriptors match in 45
+// instead of 47 us.)
+__global__ void expand_two_kernel(const uint32_t* __restrict__ q, int64_t qwords, const uint32_t* __restrict__ t,
+                                  int64_t twords, uint4* __restrict__ out, int32_t* __restrict__ counters,
+                                  int32_t ncounters) {
+    griddep_wait();
+    griddep_launch_dependents();
+    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (i < ncounters) counters[i] = 0;
+    if (i < qwords)
+        out[i] = expand_word_e2m1(q[i]);
+    else if (i < qwords + twords)
+        out[i] = expand_word_e2m1(t[i - qwords]);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -756,14 +809,16 @@ cudaError_t launch_expand(const uint8_t* desc, int64_t n, uint8_t* out, cudaStre
                           reinterpret_cast<const uint32_t*>(desc), nwords, reinterpret_cast<uint4*>(out));
 }
 
-// Fills tiles, unit offsets, query-tile prefixes and the block split.  problems[i]
+int64_t match_tc_tiles(int64_t nq) { return (nq + kRowsQ - 1) / kRowsQ; }
+
+// Fills tiles, unit offsets, query-tile prefixes and the split over the block pairs.  problems[i]
 // must have q_row0, t_row0, nq, nt and out0 set.
-void plan_match_batch(MatchBatch* b, int count, int64_t max_grid) {
+void plan_match_batch(MatchBatch* b, int count, int64_t max_sms) {
     b->count = count;
     int64_t units = 0, g = 0, queries = 0;
     for (int i = 0; i < count; ++i) {
         MatchProblem& P = b->p[i];
-        P.mt = (P.nq + kRowsQ - 1) / kRowsQ;
+        P.mt = static_cast<int32_t>(match_tc_tiles(P.nq));
         P.ntl = P.nq > 0 ? (P.nt + kColsB - 1) / kColsB : 0;
         P.unit0 = units;
         P.g0 = static_cast<int32_t>(g);
@@ -774,12 +829,13 @@ void plan_match_batch(MatchBatch* b, int count, int64_t max_grid) {
     b->units = units;
     b->tiles = static_cast<int32_t>(g);
     b->queries = queries;
-    b->grid = units < max_grid ? units : max_grid;
+    const int64_t pairs = max_sms / 2 > 0 ? max_sms / 2 : 1;
+    b->grid = units < pairs ? units : pairs;
     // whole query tiles per share when there are enough of them to balance the
     // blocks (the block that walks a whole tile writes its matches directly, and a
     // tile's walk pays its start-up -- the first units' top-two updates -- once);
     // not when some problem has queries but no train rows (its tiles have no unit)
-    bool whole = g >= kWholeTilesPerBlock * b->grid;
+    bool whole = g >= kWholeTilesPerPair * b->grid;
     for (int i = 0; i < count; ++i)
         if (b->p[i].nq > 0 && b->p[i].ntl == 0) whole = false;
     b->whole_tiles = whole ? 1 : 0;
@@ -787,18 +843,20 @@ void plan_match_batch(MatchBatch* b, int count, int64_t max_grid) {
 
 // Slots g + c' + p (G - 1) (UnitIter): tiles + count (G - 1) of them.
 static size_t partial_record_bytes(const MatchBatch& b) {
-    return static_cast<size_t>(b.tiles + static_cast<int64_t>(b.count) * b.grid + 1) * kRowsP * 16;
+    const int64_t shares = b.grid > 0 ? b.grid - 1 : 0;
+    return static_cast<size_t>(b.tiles + static_cast<int64_t>(b.count) * shares) * kRowsP * 16;
 }
 
 size_t match_tc_partial_bytes(const MatchBatch& b) { return partial_record_bytes(b); }
 
-size_t match_tc_counter_bytes(int64_t tiles) { return align_up(static_cast<size_t>(tiles) * 4, 256); }
+// A counter for each half of a query tile.
+size_t match_tc_counter_bytes(int64_t tiles) { return align_up(static_cast<size_t>(tiles) * 8, 256); }
 
 // A launch over `problems` problems with `queries` query rows in total has at most
-// queries / 128 + problems query tiles and at most `sms` blocks.
+// queries / 256 + problems query tiles and at most `sms` / 2 block pairs.
 size_t match_tc_partial_bound(int64_t queries, int64_t problems, int64_t sms) {
     const int64_t tiles = queries / kRowsQ + problems;
-    return static_cast<size_t>(tiles + problems * sms + 1) * kRowsP * 16 + match_tc_counter_bytes(tiles) + 512;
+    return static_cast<size_t>(tiles + problems * (sms / 2 + 1)) * kRowsP * 16 + match_tc_counter_bytes(tiles) + 512;
 }
 
 size_t match_tc_batch_scratch_bytes(int64_t rows, const MatchBatch& b, int64_t counter_tiles) {
@@ -843,7 +901,7 @@ static cudaError_t launch_match_np(const MatchBatch& full, const CUtensorMap& ma
     shrink(full, b);
     cudaError_t e = cudaSuccess;
     if (b->units > 0)
-        e = launch_chained(match_tc_kernel<NP>, dim3(static_cast<unsigned>(b->grid)), dim3(kThreads), kSmemBytes,
+        e = launch_chained(match_tc_kernel<NP>, dim3(static_cast<unsigned>(2 * b->grid)), dim3(kThreads), kSmemBytes,
                            stream, mapq, mapt, *b, partials, tile_cnt, out, flags);
     if (e == cudaSuccess && !tile_cnt && !b->whole_tiles && b->queries > 0) {
         const int threads = 256;
@@ -859,15 +917,15 @@ cudaError_t launch_match_tc_rows(const MatchBatch& b, const uint8_t* exp, int64_
                                  cudaStream_t stream) {
     if (b.queries == 0) return cudaSuccess;
     CUtensorMap mapq, mapt;
-    if (b.units > 0 && !(make_map(&mapq, exp, rows, kRowsA) && make_map(&mapt, exp, rows, kColsB)))
+    if (b.units > 0 && !(make_map(&mapq, exp, rows, kRowsA) && make_map(&mapt, exp, rows, kRowsB)))
         return cudaErrorInvalidValue;
-    // a short launch (at most kFusedUnitsPerBlock units per block) combines each query
+    // a short launch (at most kFusedUnitsPerPair units per block) combines each query
     // tile's records itself, which saves the merge launch; a long one leaves them to
     // match_merge_kernel, because the combine at a tile's end (a fence and an atomic
     // round trip per block) holds the epilogue while the MMAs can run only an
     // accumulator's worth ahead.  Neither when some problem has queries but no train
     // rows (its tiles have no unit, so no block visits them).
-    bool fused = b.units > 0 && tile_cnt != nullptr && b.units <= kFusedUnitsPerBlock * b.grid;
+    bool fused = b.units > 0 && tile_cnt != nullptr && b.units <= kFusedUnitsPerPair * b.grid;
     for (int i = 0; i < b.count; ++i)
         if (b.p[i].nq > 0 && b.p[i].ntl == 0) fused = false;
     if (!fused) tile_cnt = nullptr;
@@ -917,10 +975,13 @@ cudaError_t launch_match_tc(const latch_context* ctx, const uint8_t* q, int32_t 
     uint8_t* base = static_cast<uint8_t*>(scratch);
     cudaError_t e = cudaSuccess;
     if (b->units > 0) {
-        // the arrival counters are cleared ahead of the kernels, off their dependency chain
-        e = cudaMemsetAsync(match_tc_batch_counters(scratch, nq + nt), 0, match_tc_counter_bytes(b->tiles), stream);
-        if (e == cudaSuccess) e = launch_expand(q, nq, base, stream);
-        if (e == cudaSuccess) e = launch_expand(t, nt, base + static_cast<size_t>(nq) * kKBytes, stream);
+        const int64_t qwords = static_cast<int64_t>(nq) * kDescWords, twords = static_cast<int64_t>(nt) * kDescWords;
+        const int32_t ncounters = 2 * b->tiles;  // fewer than the query words
+        const int threads = 256;
+        e = launch_chained(expand_two_kernel, dim3(static_cast<unsigned>((qwords + twords + threads - 1) / threads)),
+                           dim3(threads), 0, stream, reinterpret_cast<const uint32_t*>(q), qwords,
+                           reinterpret_cast<const uint32_t*>(t), twords, reinterpret_cast<uint4*>(base),
+                           match_tc_batch_counters(scratch, static_cast<int64_t>(nq) + nt), ncounters);
     }
     if (e == cudaSuccess) e = launch_match_tc_batch(*b, nq + nt, b->tiles, scratch, out, ctx->d_flags, stream);
     delete b;

@@ -99,6 +99,17 @@ __device__ __forceinline__ bool mbar_wait_sleep(uint64_t* bar, uint32_t parity, 
     }
 }
 
+// One lane of a converged warp (the same one every time).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t e;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(e));
+    return e != 0;
+}
+
 // 2-D tiled TMA load into shared memory, completing tx bytes on `bar`.
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int32_t x, int32_t y, uint64_t* bar) {
     asm volatile(
@@ -130,12 +141,6 @@ __device__ __forceinline__ void sts_u32(uint32_t addr, uint32_t v) {
     asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
-// Named barrier `kId` of `kCount` threads (memory ordering among them).
-template <int kId, int kCount>
-__device__ __forceinline__ void bar_sync() {
-    asm volatile("bar.sync %0, %1;" ::"n"(kId), "n"(kCount) : "memory");
-}
-
 // The same with a run-time barrier id.
 __device__ __forceinline__ void bar_sync_id(int id, int count) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
@@ -152,28 +157,41 @@ __device__ __forceinline__ void set_max_regs_inc() {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegs));
 }
 
-// AND of `v` over the `kCount` threads meeting at named barrier `kId` (a barrier
-// with memory ordering among them, like __syncthreads_and for a part of a block).
-template <int kId, int kCount>
-__device__ __forceinline__ bool bar_and(bool v) {
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 q, %1, 0;\n\t"
-        "bar.red.and.pred p, %2, %3, q;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(r)
-        : "r"(static_cast<uint32_t>(v)), "n"(kId), "n"(kCount)
-        : "memory");
-    return r != 0;
-}
-
 // 16-byte asynchronous global -> shared copy (L2 only); completion by cp_async_wait_all
 // in the issuing thread.
 __device__ __forceinline__ void cp_async_16(void* dst_smem, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst_smem)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// ---- block pairs (clusters of two) ----------------------------------------------
+
+// Every thread of both blocks (memory ordering among them, shared memory included).
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Shared-memory address `addr` of this block in block `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+
+// Arrives on a barrier given by its cluster address.
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+
+// 2-D tiled TMA load into this block's shared memory, completing tx bytes on a barrier of
+// either block of the pair (its cluster address).
+__device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* map, int32_t x, int32_t y, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+        "[%4];" ::"r"(smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
+        : "memory");
+}
 
 // ---- tcgen05 -------------------------------------------------------------------
 
@@ -191,46 +209,41 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// D[tmem] (+)= (A[smem] x scale_A) * (B[smem] x scale_B)^T with 4-bit E2M1 operands
-// (two per byte, K = 64 per instruction) and per-32-value block scales read from TMEM
-// (sfa / sfb: TMEM addresses of the scale columns), fp32 accumulate.
-__device__ __forceinline__ void mma_mxf4(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                         uint32_t sfa, uint32_t sfb, uint32_t accumulate) {
+// D[tmem] (+)= (A[smem] x scale_A) * (B[smem] x scale_B)^T with 4-bit E2M1 operands (two per
+// byte) and per-32-value block scales read from TMEM (sfa / sfb: TMEM addresses of the
+// scale columns), fp32 accumulate, by a block pair, issued by its first block: D's and A's
+// rows are split over the two blocks (M / 2 each), and so are B's (N / 2 each); K by the
+// instruction descriptor (64 or 96).
+__device__ __forceinline__ void mma_mxf4_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                              uint32_t sfa, uint32_t sfb, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %6, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], %1, %2, %3, [%4], [%5], p;\n\t}" ::"r"(
-            d_tmem),
+        "tcgen05.mma.cta_group::2.kind::mxf4.block_scale.block32 [%0], %1, %2, %3, [%4], [%5], p;\n\t}" ::"r"(d_tmem),
         "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(sfa), "r"(sfb), "r"(accumulate)
         : "memory");
 }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, BF16 operands, fp32 accumulate.
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                         uint32_t accumulate) {
+// Arrive on the barrier at `bar`'s offset in both blocks of the pair once all previously
+// issued pair MMAs of this thread complete.
+__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+            smem_u32(bar)),
+        "h"(static_cast<uint16_t>(3))
         : "memory");
 }
 
-// Shared-memory descriptor: K-major operand without swizzle, core matrices of 8 rows
-// x 16 bytes (128 contiguous bytes); `lbo` bytes between core matrices along K,
-// `sbo` bytes between 8-row groups.
-__device__ __forceinline__ uint64_t umma_desc_noswizzle(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-    uint64_t d = 0;
-    d |= static_cast<uint64_t>((addr & 0x3FFFFu) >> 4);
-    d |= static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16;
-    d |= static_cast<uint64_t>((sbo >> 4) & 0x3FFFu) << 32;
-    d |= static_cast<uint64_t>(1) << 46;  // descriptor version (sm_100 family); layout type 0: no swizzle
-    return d;
+// TMEM of a block pair whose MMAs span it: one warp of each block.
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t* dst_smem, uint32_t ncols) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)),
+                 "r"(ncols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
 }
-
-// Makes this thread's generic-proxy shared-memory writes visible to the async proxy
-// (tensor-core operand reads, TMA).
-__device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
 
 // Stores `v` into 8 consecutive 32-bit TMEM columns of 32 lanes: thread i of the
 // warp writes lane (taddr.lane + i), columns taddr.col .. +7.
@@ -259,40 +272,8 @@ __device__ __forceinline__ void tmem_st_32x32b_x2(uint32_t taddr, uint32_t a, ui
 
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// Arrive on `bar` once all previously issued tcgen05.mma of this thread complete.
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-}
-
-// 32 lanes x 32 consecutive 32-bit columns: thread i of the warp gets lane
-// (taddr.lane + i), columns taddr.col .. +31.
-__device__ __forceinline__ void tmem_ld_32x32b_x32(uint32_t taddr, uint32_t (&v)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-        : "r"(taddr)
-        : "memory");
-}
-
-// 32 lanes x 16 consecutive 32-bit columns.
-__device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t (&v)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-        : "r"(taddr)
-        : "memory");
-}
-
-// 32 lanes x 8 consecutive 32-bit columns.
-// As tmem_ld_32x32b_x16, and *mx = the largest of the thread's 16 values (as f32).
+// 32 lanes x 16 consecutive 32-bit columns, and mx = the largest of the thread's 16
+// values (as f32).
 __device__ __forceinline__ void tmem_ld_red_max_32x32b_x16(uint32_t taddr, uint32_t (&v)[16], float& mx) {
     asm volatile(
         "tcgen05.ld.red.sync.aligned.32x32b.x16.max.f32 "
@@ -324,13 +305,8 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t addr) {
     return d;
 }
 
-// Instruction descriptor for kind::f16: A, B = BF16, D = F32, both K-major.
-__host__ __device__ constexpr uint32_t idesc_bf16_f32(int m, int n) {
-    return (1u << 4)                                   // D format F32
-           | (1u << 7) | (1u << 10)                    // A, B = BF16
-           | (static_cast<uint32_t>(n >> 3) << 17)     // N / 8
-           | (static_cast<uint32_t>(m >> 4) << 24);    // M / 16
-}
+// K = 96 instead of 64 in an instruction descriptor of kind::mxf4 (sm_103a).
+constexpr uint32_t kIdescK96 = 1u << 31;
 
 // Instruction descriptor for kind::mxf4 (block-scaled): A, B = E2M1, scales UE8M0,
 // D = F32, both K-major, scale-factor byte ids 0.
