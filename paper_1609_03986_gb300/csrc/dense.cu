@@ -8,9 +8,9 @@
 // with A = I(p + a - 24 + d), C1, C2 likewise (Eq. 1; one product image per triplet,
 // then a separable 7x7 box sum; all exact in int32, |box| <= 49 * 255 * 510).
 //
-// dense_extract_kernel: one block per 32x32-pixel tile; the image region under the
-// tile and every window (79 x 79 bytes, 0 outside the image) is staged once in shared
-// memory.  Per round two triplets t and t + 256:
+// dense_extract_kernel: one block per 32x32-pixel tile and share of the triplets; the image
+// region under the tile and every window (79 x 79 bytes, 0 outside the image) is staged
+// once in shared memory.  Per round two triplets, from the two halves of the share:
 //   phase A (304 threads, 2 x 38 rows x 4 segments): a thread forms the product image
 //            along 14 pixels of one row (each patch's 14 bytes from five aligned
 //            words) and writes 8 horizontal 7-sums;
@@ -49,7 +49,8 @@ constexpr int kSegs = 4;                        // 8-pixel segments per row / co
 constexpr int kAThreads = kHRows * kSegs;       // 152 per triplet
 constexpr int kBThreads = kTile * kSegs;        // 128 per triplet
 constexpr int kDenseThreads = 320;
-constexpr int kHalfBits = kBits / 2;            // triplets t and t + 256 share a round
+constexpr int kBlocksPerSm = 6;
+constexpr int kMaxShares = 8;                   // a share is at least two descriptor words
 
 struct DenseTriplets {
     latch_triplet t[kBits];
@@ -62,13 +63,14 @@ struct DenseSmem {
     alignas(16) int32_t h[2][2][kHRows][kHPitch];  // [round parity][triplet slot][row][column]
 };
 
-__global__ void __launch_bounds__(kDenseThreads) dense_extract_kernel(const uint8_t* __restrict__ img, int width,
-                                                                      int height, int64_t pitch,
+__global__ void __launch_bounds__(kDenseThreads, 3) dense_extract_kernel(const uint8_t* __restrict__ img, int width,
+                                                                      int height, int64_t pitch, int half,
                                                                       const __grid_constant__ DenseTriplets tr,
                                                                       uint32_t* __restrict__ out) {
     __shared__ __align__(16) DenseSmem S;
     const int tid = threadIdx.x;
     const int x0 = blockIdx.x * kTile, y0 = blockIdx.y * kTile;
+    const int first = blockIdx.z * 2 * half;  // the share's triplets: [first, first + 2 half)
     griddep_wait();
     griddep_launch_dependents();
     // stage the region [x0 - 24, x0 + 55) x [y0 - 24, y0 + 55); samples outside read 0
@@ -81,8 +83,8 @@ __global__ void __launch_bounds__(kDenseThreads) dense_extract_kernel(const uint
     }
     // patch at window point (x, y) of the pixel at tile offset (fx, fy): staged pixel
     // (fx + x - 3 + dx, fy + y - 3 + dy) for dx, dy in 0..6 -- the thread's base plus off
-    for (int t = tid; t < kBits; t += kDenseThreads) {
-        const uint8_t* c = &tr.t[t].ax;
+    for (int t = tid; t < 2 * half; t += kDenseThreads) {
+        const uint8_t* c = &tr.t[first + t].ax;
         for (int p = 0; p < 3; ++p)
             S.off[p][t] = static_cast<uint16_t>((c[2 * p + 1] - kPatchR) * kRegionPitch + (c[2 * p] - kPatchR));
     }
@@ -114,7 +116,7 @@ __global__ void __launch_bounds__(kDenseThreads) dense_extract_kernel(const uint
         return static_cast<int>(__byte_perm(y[i >> 2], 0u, 0x4440u | static_cast<uint32_t>(i & 3)));
     };
     auto phase_a = [&](int k) {
-        const int t = ja * kHalfBits + k;
+        const int t = ja * half + k;
         uint32_t ya[4], y1[4], y2[4];
         load14(abase + S.off[0][t], ya);
         load14(abase + S.off[1][t], y1);
@@ -136,7 +138,7 @@ __global__ void __launch_bounds__(kDenseThreads) dense_extract_kernel(const uint
 
     if (tid < 2 * kAThreads) phase_a(0);
     __syncthreads();
-    for (int k = 0; k < kHalfBits; ++k) {
+    for (int k = 0; k < half; ++k) {
         if (tid < 2 * kBThreads) {
             const int32_t* hc = &S.h[k & 1][jb][kTile / kSegs * sb][cb];
             int hv[14];
@@ -151,8 +153,8 @@ __global__ void __launch_bounds__(kDenseThreads) dense_extract_kernel(const uint
                 bits[j] |= static_cast<uint32_t>(v > 0) << b;
             }
             if (b == 31) {
-                // descriptor word (jb * 256 + k) / 32 of the segment's 8 pixels
-                const int w = jb * (kHalfBits / 32) + (k >> 5);
+                // the descriptor word of triplet first + jb half + k, of the segment's 8 pixels
+                const int w = (first + jb * half + k) >> 5;
                 const int x = x0 + cb;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
@@ -162,7 +164,7 @@ __global__ void __launch_bounds__(kDenseThreads) dense_extract_kernel(const uint
                 }
             }
         }
-        if (k + 1 < kHalfBits && tid < 2 * kAThreads) phase_a(k + 1);
+        if (k + 1 < half && tid < 2 * kAThreads) phase_a(k + 1);
         __syncthreads();
     }
 }
@@ -257,10 +259,15 @@ cudaError_t launch_dense_extract(const latch_context* ctx, const latch_image* im
                                  cudaStream_t stream) {
     DenseTriplets tr;
     for (int t = 0; t < kBits; ++t) tr.t[t] = ctx->h_trip[t];
-    const dim3 grid(static_cast<unsigned>((img->width + kTile - 1) / kTile),
-                    static_cast<unsigned>((img->height + kTile - 1) / kTile));
+    const int tx = (img->width + kTile - 1) / kTile, ty = (img->height + kTile - 1) / kTile;
+    // An SM holds three blocks; the triplets are shared out until there are about six per SM,
+    // so that the last round of blocks is short (640x480, 300 tiles: 343 us with one share,
+    // 234, 228 and 234 us with 2, 4 and 8, which stage the region more often).
+    int shares = 1;
+    while (shares < kMaxShares && static_cast<int64_t>(tx) * ty * shares < kBlocksPerSm * ctx->sm_count) shares *= 2;
+    const dim3 grid(static_cast<unsigned>(tx), static_cast<unsigned>(ty), static_cast<unsigned>(shares));
     return launch_chained(dense_extract_kernel, grid, dim3(kDenseThreads), 0, stream, img->data, img->width,
-                          img->height, img->pitch, tr, reinterpret_cast<uint32_t*>(d_out));
+                          img->height, img->pitch, kBits / (2 * shares), tr, reinterpret_cast<uint32_t*>(d_out));
 }
 
 static cudaError_t set_dense_match_attributes() {
