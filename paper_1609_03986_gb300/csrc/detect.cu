@@ -51,19 +51,23 @@ constexpr double kPi = 3.141592653589793;
 __constant__ int8_t c_circle[16][2] = {{0, -3}, {1, -3}, {2, -2}, {3, -1}, {3, 0},  {3, 1},  {2, 2},  {1, 3},
                                        {0, 3},  {-1, 3}, {-2, 2}, {-3, 1}, {-3, 0}, {-3, -1}, {-2, -2}, {-1, -3}};
 
+// Whether the pixel at tile position (tx, ty) can be a corner: a run of 9 covers two
+// neighbouring compass points (0, 4, 8, 12).
+__device__ __forceinline__ bool fast_candidate(const uint8_t (*tile)[kTileD], int tx, int ty, int t) {
+    const int p = tile[ty][tx];
+    const int n0 = tile[ty - 3][tx], n4 = tile[ty][tx + 3], n8 = tile[ty + 3][tx], n12 = tile[ty][tx - 3];
+    const int hi = p + t, lo = p - t;
+    // two neighbouring compass points are one of (0, 8) and one of (4, 12)
+    const bool bright = max(n0, n8) > hi && max(n4, n12) > hi;
+    const bool dark = min(n0, n8) < lo && min(n4, n12) < lo;
+    return bright || dark;
+}
+
 // FAST score of the pixel at tile position (tx, ty): the best arc of 9 over both
 // polarities, max over arcs of min over the arc of (I_k - I_p) (bright) or of
 // (I_p - I_k) (dark), minus 1; 0 when below t.
 __device__ __forceinline__ int fast_score(const uint8_t (*tile)[kTileD], int tx, int ty, int t) {
     const int p = tile[ty][tx];
-    // quick rejection: a run of 9 covers two neighbouring compass points (0, 4, 8, 12)
-    const int n0 = tile[ty - 3][tx], n4 = tile[ty][tx + 3], n8 = tile[ty + 3][tx], n12 = tile[ty][tx - 3];
-    const int hi = p + t, lo = p - t;
-    const bool b0 = n0 > hi, b4 = n4 > hi, b8 = n8 > hi, b12 = n12 > hi;
-    const bool d0 = n0 < lo, d4 = n4 < lo, d8 = n8 < lo, d12 = n12 < lo;
-    const bool bright = (b0 && b4) || (b4 && b8) || (b8 && b12) || (b12 && b0);
-    const bool dark = (d0 && d4) || (d4 && d8) || (d8 && d12) || (d12 && d0);
-    if (!bright && !dark) return 0;
     int d[16];
 #pragma unroll
     for (int k = 0; k < 16; ++k) d[k] = static_cast<int>(tile[ty + c_circle[k][1]][tx + c_circle[k][0]]) - p;
@@ -89,6 +93,22 @@ __device__ __forceinline__ int fast_score(const uint8_t (*tile)[kTileD], int tx,
     }
     const int s = max(best_b, best_d) - 1;
     return s >= t ? s : 0;
+}
+
+// round_half_away(atan2(m01, m10) * 16 / pi) mod 32 in FP64.  FP32 decides it wherever its
+// value is at least 1e-3 away from a half-integer (its error, with moments below 2^24, is
+// below 1e-5; the FP64 value then rounds to the same integer), which spares all but about
+// 0.2% of the keypoints the FP64 arithmetic: this GPU has little of it, and it took most
+// of the detection's time (about 430 us for a 4000x3000 image's three levels, 162 us now).
+__device__ __forceinline__ int angle_bin(int m10, int m01) {
+    const float t = atan2f(static_cast<float>(m01), static_cast<float>(m10)) * static_cast<float>(16.0 / kPi);
+    const float r = rintf(t);
+    int b = static_cast<int>(r);
+    if (!(0.5f - fabsf(t - r) > 1e-3f)) {
+        const double theta = atan2(static_cast<double>(m01), static_cast<double>(m10));
+        b = static_cast<int>(round(theta * 16.0 / kPi));
+    }
+    return ((b % 32) + 32) % 32;
 }
 
 struct DetectLevel {
@@ -117,10 +137,12 @@ __device__ __forceinline__ int level_of_cell(const DetectParams& prm, int cell) 
     return l;
 }
 
-__global__ void __launch_bounds__(kDetThreads) detect_cells_kernel(const DetectParams prm, int32_t* __restrict__ counts,
+__global__ void __launch_bounds__(kDetThreads, 6) detect_cells_kernel(const DetectParams prm, int32_t* __restrict__ counts,
                                                                    uint16_t* __restrict__ slots) {
     __shared__ __align__(16) uint8_t tile[kTileD][kTileD];
     __shared__ uint8_t sc[kApron][kApron];
+    __shared__ uint16_t cand[kApron * kApron];
+    __shared__ int ncand;
     __shared__ uint16_t keep[kMaxPerCell];
     __shared__ int warp_tot[kDetThreads / 32];
     griddep_wait();
@@ -159,14 +181,35 @@ __global__ void __launch_bounds__(kDetThreads) detect_cells_kernel(const DetectP
         }
         *reinterpret_cast<uint4*>(&tile[r][16 * q]) = v;
     }
+    if (threadIdx.x == 0) ncand = 0;
     __syncthreads();
-    // ---- scores of pixels x0-1 .. x0+32, y0-1 .. y0+32 (0 where the circle leaves the image) ----
-    for (int i = threadIdx.x; i < kApron * kApron; i += kDetThreads) {
-        const int ay = i / kApron, ax = i % kApron;
-        const int gx = x0 - 1 + ax, gy = y0 - 1 + ay;
-        int s = 0;
-        if (gx >= 3 && gy >= 3 && gx < W - 3 && gy < H - 3) s = fast_score(tile, ax + kHaloD - 1, ay + kHaloD - 1, prm.t);
-        sc[ay][ax] = static_cast<uint8_t>(s);
+    // ---- scores of pixels x0-1 .. x0+32, y0-1 .. y0+32 (0 where the circle leaves the image):
+    // first the candidates, then the scores of the candidates side by side.  Scored where they
+    // lie, nearly every warp holds a candidate and runs the whole test for it (a 4000x3000
+    // image's three levels: 223 us for the whole detection, 162 us this way). ----
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i0 = 0; i0 < kApron * kApron; i0 += kDetThreads) {
+        const int i = i0 + threadIdx.x;
+        bool c = false;
+        if (i < kApron * kApron) {
+            const int ay = i / kApron, ax = i - ay * kApron;
+            const int gx = x0 - 1 + ax, gy = y0 - 1 + ay;
+            c = gx >= 3 && gy >= 3 && gx < W - 3 && gy < H - 3 &&
+                fast_candidate(tile, ax + kHaloD - 1, ay + kHaloD - 1, prm.t);
+            sc[ay][ax] = 0;
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, c);
+        if (m) {
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&ncand, __popc(m));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (c) cand[at + __popc(m & ((1u << lane) - 1u))] = static_cast<uint16_t>(i);
+        }
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < ncand; k += kDetThreads) {
+        const int i = cand[k], ay = i / kApron, ax = i - ay * kApron;
+        sc[ay][ax] = static_cast<uint8_t>(fast_score(tile, ax + kHaloD - 1, ay + kHaloD - 1, prm.t));
     }
     __syncthreads();
     // ---- suppression: thread = 4 consecutive pixels of one cell row (raster order) ----
@@ -186,7 +229,6 @@ __global__ void __launch_bounds__(kDetThreads) detect_cells_kernel(const DetectP
         mask |= static_cast<uint32_t>(k) << j;
     }
     // exclusive scan of the per-thread counts (thread order = raster order)
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int cnt = __popc(mask);
     int incl = cnt;
 #pragma unroll
@@ -225,16 +267,18 @@ __global__ void __launch_bounds__(kDetThreads) detect_cells_kernel(const DetectP
         m10 = __reduce_add_sync(0xffffffffu, m10);
         m01 = __reduce_add_sync(0xffffffffu, m01);
         if (lane == 0) {
-            const double theta = atan2(static_cast<double>(m01), static_cast<double>(m10));
-            const int b = static_cast<int>(round(theta * 16.0 / kPi));
-            const int bin = ((b % 32) + 32) % 32;
+            const int bin = angle_bin(m10, m01);
             slots[static_cast<int64_t>(cell) * kMaxPerCell + i] = static_cast<uint16_t>((bin << 10) | keep[i]);
         }
     }
     if (threadIdx.x == 0) counts[cell] = total;
 }
 
-// Exclusive scan of the cell counts in place (offsets), total -> *d_count.
+// Exclusive scan of the cell counts in place (offsets), total -> *d_count.  One block: a
+// thread takes 16 consecutive cells per pass (four 16-byte loads), so that the cells of a
+// large image are a pass or two of global latency.
+constexpr int kScanItems = 16;
+
 __global__ void __launch_bounds__(1024) detect_scan_kernel(int32_t* __restrict__ counts, int32_t ncells,
                                                            int32_t* __restrict__ d_count) {
     __shared__ int part[32];
@@ -242,35 +286,50 @@ __global__ void __launch_bounds__(1024) detect_scan_kernel(int32_t* __restrict__
     griddep_launch_dependents();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int carry = 0;
-    for (int c0 = 0; c0 < ncells; c0 += 8 * 1024) {
-        const int c = c0 + 8 * threadIdx.x;
-        int v[8], sum = 0;
+    for (int c0 = 0; c0 < ncells; c0 += kScanItems * 1024) {
+        const int c = c0 + kScanItems * static_cast<int>(threadIdx.x);
+        const bool whole = c + kScanItems <= ncells;
+        int v[kScanItems], sum = 0;
+        if (whole) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            v[q] = c + q < ncells ? counts[c + q] : 0;
-            sum += v[q];
-        }
-        int incl = sum;
+            for (int q = 0; q < kScanItems / 4; ++q)
+                *reinterpret_cast<int4*>(&v[4 * q]) = reinterpret_cast<const int4*>(counts + c)[q];
+        } else {
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int x = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += x;
+            for (int q = 0; q < kScanItems; ++q) v[q] = c + q < ncells ? counts[c + q] : 0;
         }
-        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kScanItems; ++q) sum += v[q];
+        auto scan = [&](int x) {  // inclusive, over the warp
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            return x;
+        };
+        const int incl = scan(sum);
         if (lane == 31) part[warp] = incl;
         __syncthreads();
-        int run = carry + incl - sum, tile_total = 0;
-        for (int w = 0; w < 32; ++w) {
-            run += w < warp ? part[w] : 0;
-            tile_total += part[w];
-        }
+        const int all = scan(part[lane]);  // every warp scans the warps' totals for itself
+        int run = carry + incl - sum + (warp ? __shfl_sync(0xffffffffu, all, warp - 1) : 0);
+        carry += __shfl_sync(0xffffffffu, all, 31);
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-            if (c + q < ncells) {
-                counts[c + q] = run;
-                run += v[q];
-            }
-        carry += tile_total;
+        for (int q = 0; q < kScanItems; ++q) {
+            const int n = v[q];
+            v[q] = run;
+            run += n;
+        }
+        if (whole) {
+#pragma unroll
+            for (int q = 0; q < kScanItems / 4; ++q)
+                reinterpret_cast<int4*>(counts + c)[q] = *reinterpret_cast<const int4*>(&v[4 * q]);
+        } else {
+#pragma unroll
+            for (int q = 0; q < kScanItems; ++q)
+                if (c + q < ncells) counts[c + q] = v[q];
+        }
+        __syncthreads();  // the totals are read before the next pass writes them
     }
     if (threadIdx.x == 0) *d_count = carry;
 }
@@ -310,16 +369,20 @@ __global__ void __launch_bounds__(256) detect_expand_kernel(const DetectParams p
     }
 }
 
-// Level images of the levels with scale != 1: one thread per 16 output bytes of a
-// row, rows of all levels in one grid (row r of the launch is level `lev`'s row
-// r - row0[lev]).  out(x, y) = base(rha(s x), rha(s y)).
+// Level images of the levels with scale != 1: one thread per 16 output columns of
+// kLevelRows rows, row groups of all levels in one grid (group r of the launch is level
+// `lev`'s group r - row0[lev]).  out(x, y) = base(rha(s x), rha(s y)).  The FP64 products
+// and roundings of the columns bound the kernel when every row computed them (74 us for
+// the two levels of a 4000x3000 image); the rows of a group share them.
+constexpr int kLevelRows = 8;
+
 struct ResampleParams {
     const uint8_t* base;
     int64_t base_pitch;
     uint8_t* out[kMaxDetectLevels];
     int64_t pitch[kMaxDetectLevels];
-    int32_t width[kMaxDetectLevels];
-    int32_t row0[kMaxDetectLevels + 1];  // first launch row of each level; row0[n] = rows of all levels
+    int32_t width[kMaxDetectLevels], height[kMaxDetectLevels];
+    int32_t row0[kMaxDetectLevels + 1];  // first row group of each level; row0[n] = groups of all levels
     double scale[kMaxDetectLevels];
     int32_t n;
     int32_t chunks;  // 16-byte chunks per launch row: those of the widest level
@@ -334,20 +397,25 @@ __global__ void __launch_bounds__(256) pyramid_level_kernel(const ResampleParams
     if (row >= prm.row0[prm.n]) return;
     int l = 0;
     while (l + 1 < prm.n && prm.row0[l + 1] <= row) ++l;
-    const int y = static_cast<int>(row - prm.row0[l]);
+    const int y0 = static_cast<int>(row - prm.row0[l]) * kLevelRows;
     const int x0 = static_cast<int>(gid % chunks_per_row) * 16;
-    const int w = prm.width[l];
+    const int w = prm.width[l], h = prm.height[l];
     if (x0 >= w) return;
     const double s = prm.scale[l];
-    const uint8_t* src = prm.base + static_cast<int64_t>(round(s * static_cast<double>(y))) * prm.base_pitch;
-    union {
-        uint4 v;
-        uint8_t b[16];
-    } u;
+    int32_t sx[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-        u.b[i] = x0 + i < w ? src[static_cast<int64_t>(round(s * static_cast<double>(x0 + i)))] : 0;
-    *reinterpret_cast<uint4*>(prm.out[l] + static_cast<int64_t>(y) * prm.pitch[l] + x0) = u.v;
+        sx[i] = x0 + i < w ? static_cast<int32_t>(round(s * static_cast<double>(x0 + i))) : -1;
+    for (int y = y0; y < y0 + kLevelRows && y < h; ++y) {
+        const uint8_t* src = prm.base + static_cast<int64_t>(round(s * static_cast<double>(y))) * prm.base_pitch;
+        union {
+            uint4 v;
+            uint8_t b[16];
+        } u;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) u.b[i] = sx[i] >= 0 ? src[sx[i]] : 0;
+        *reinterpret_cast<uint4*>(prm.out[l] + static_cast<int64_t>(y) * prm.pitch[l] + x0) = u.v;
+    }
 }
 
 }  // namespace
@@ -423,8 +491,9 @@ cudaError_t launch_detect(const latch_image* img, const double* scales, const in
         rs.out[k] = base + off;
         rs.pitch[k] = L.pitch;
         rs.width[k] = L.width;
+        rs.height[k] = L.height;
         rs.scale[k] = L.scale;
-        rs.row0[k + 1] = rs.row0[k] + L.height;
+        rs.row0[k + 1] = rs.row0[k] + (L.height + kLevelRows - 1) / kLevelRows;
         rs.chunks = std::max<int32_t>(rs.chunks, (L.width + 15) / 16);
         off += (static_cast<size_t>(L.height) * L.pitch + 255) / 256 * 256;
     }
