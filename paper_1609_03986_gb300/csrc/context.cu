@@ -116,10 +116,18 @@ static latch_status upload_scales(latch_context* ctx, const double* scales, int 
     return LATCH_OK;
 }
 
-// Matching path for AUTO: the tensor-core path once the pair count amortises its
-// operand expansion and merge launches (threshold set by latch_autotune).
+// Matching path for AUTO: the tensor cores from tensor_min_pairs pairs on
+// (latch_autotune, latch_set_tuning).  At its default value they also take smaller
+// problems of more than one CUDA-core train tile (256 rows): a block of the CUDA cores
+// needs about 18 us for a tile's rows whatever the query count and merges the tiles in a
+// second launch, the tensor path 12 us with its expansion (300 x 300: 18.5 against 11.8
+// us, 2,000 x 2,000: 28.4 / 14.5, 100 x 10,000: 30.8 / 24.1; up to 256 rows 10,000 x 100:
+// 10.3 / 12.0, 50,000 x 20: 8.5 / 24.0).  Beyond 65,536 train rows the pair count decides
+// alone: the path's scratch is 256 bytes per row.
 static int choose_match_path(const latch_context* ctx, int64_t nq, int64_t nt) {
-    return nq * nt >= ctx->tensor_min_pairs ? LATCH_PATH_TENSOR : LATCH_PATH_POPC;
+    if (nq * nt >= ctx->tensor_min_pairs) return LATCH_PATH_TENSOR;
+    const bool small = ctx->tensor_min_pairs == kDefaultTensorMinPairs && nt > 256 && nt <= 65536;
+    return small ? LATCH_PATH_TENSOR : LATCH_PATH_POPC;
 }
 
 // Triplet coordinates must keep every patch inside the 48x48 window: [3, 44] for the

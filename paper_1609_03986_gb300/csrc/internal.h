@@ -46,6 +46,8 @@ __device__ __forceinline__ uint4 expand_word_e2m1(uint32_t w) {
 }
 #endif
 
+constexpr int64_t kDefaultTensorMinPairs = int64_t(1) << 22;
+
 // Device-side error flags (OR-ed into ctx->d_flags).
 enum : uint32_t { kFlagBadScale = 1u, kFlagTimeout = 2u };
 
@@ -95,7 +97,7 @@ struct latch_context {
     // extraction and matching, and after matching
     cudaEvent_t* trace_ev = nullptr;
     int32_t trace_cap = 0, trace_n = 0;
-    int64_t tensor_min_pairs = int64_t(1) << 22;  // matching: AUTO uses the tensor path from here
+    int64_t tensor_min_pairs = latch::kDefaultTensorMinPairs;  // matching: AUTO uses the tensor path from here
     latch::Scratch scratch[4];           // grow-only: CUDA-core matching, tensor matching, batch, detection
     // latch_batch_run_host: two staging sets used alternately, upload stream
     latch::HostStaging staging[2];

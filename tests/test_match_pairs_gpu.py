@@ -49,3 +49,23 @@ def test_splits_over_the_pairs(gpu_ctx, nq, nt):
     for f in FIELDS:
         assert np.array_equal(got[f], want[f]), f
     gpu_ctx.check()
+
+
+@pytest.mark.parametrize("nq", [1, 17, 300, 2000])
+@pytest.mark.parametrize("nt", [1, 255, 256, 257, 2000])
+def test_auto_route(gpu_ctx, nq, nt):
+    """LATCH_PATH_AUTO below its pair threshold: the CUDA cores up to 256 train rows, the
+    tensor cores beyond (the threshold alone once it is set), the same records on both."""
+    want = P.PATH_TENSOR if nt > 256 else P.PATH_POPC
+    assert P.hamming_match_path(gpu_ctx.handle, nq, nt) == want
+    q, t = _sets(nq, nt, nq + 3 * nt)
+    for k in (1, 2):
+        got, ref = _run(gpu_ctx, q, t, k, P.PATH_AUTO), _run(gpu_ctx, q, t, k, P.PATH_POPC)
+        for f in FIELDS:
+            assert np.array_equal(got[f], ref[f]), (k, f)
+    saved = P.latch_get_tuning(gpu_ctx.handle)
+    try:
+        P.latch_set_tuning(gpu_ctx.handle, saved["item_kps"], saved["tensor_min_pairs"] + 1)
+        assert P.hamming_match_path(gpu_ctx.handle, nq, nt) == P.PATH_POPC
+    finally:
+        P.latch_set_tuning(gpu_ctx.handle, saved["item_kps"], saved["tensor_min_pairs"])
