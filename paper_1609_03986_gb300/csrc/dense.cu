@@ -22,12 +22,12 @@
 // writes the descriptor word once.
 //
 // dense_match_kernel: one block per 16x16 pixels of image A; the descriptors of B
-// under the tile and its radius-R halo are staged in shared memory (16-byte chunks
-// swizzled so that a warp's neighbouring descriptors hit different banks); each
+// under the tile and its radius-R halo are staged in shared memory (by groups of eight
+// cells, so that a warp's neighbouring descriptors hit different banks); each
 // thread keeps its pixel's descriptor in registers and visits the (2R + 1)^2
 // candidates in raster order of B (those inside B), computing XOR + population
-// count (popc.cuh) and keeping the two best with strict comparisons, which is the
-// lowest-raster-index tie rule.
+// count (popc.cuh) and keeping the two smallest keys of distance and raster order, which
+// is the lowest-raster-index tie rule.
 #include <cstdint>
 
 #include "internal.h"
@@ -171,27 +171,41 @@ __global__ void __launch_bounds__(kDenseThreads, 3) dense_extract_kernel(const u
 
 constexpr int kMTile = 16;          // pixels of A per tile side
 constexpr int kMatchThreads = kMTile * kMTile;
+constexpr int kOrdBits = 12;        // staged row and column (less than 64 each) of a candidate
+static_assert(kMTile + 2 * LATCH_DENSE_MAX_RADIUS <= 64, "staged rows and columns take 6 bits each");
+constexpr uint32_t kNoKey = 0xffffffffu;
 
-// 16-byte chunk q of staged descriptor `cell`: chunks rotate with the cell so that
-// the 8 neighbouring descriptors read by a quarter warp fill all 32 banks.
-__device__ __forceinline__ int chunk_slot(int cell, int q) { return cell * 4 + ((q ^ (cell >> 1)) & 3); }
+// Staged descriptors: eight neighbouring cells to a group of 512 bytes, chunk q (16
+// bytes) of cell c at (c / 8) 512 + 128 q + (c % 8) 16.  Any eight neighbouring cells'
+// chunks fill all 32 banks, a candidate's four chunks are one address and constant
+// offsets, and the staging threads run along both the descriptors and the groups.
+__device__ __forceinline__ const uint4* staged_cell(const uint4* s, int c) { return s + (c >> 3) * 32 + (c & 7); }
 
+// One pixel per thread.  Keys distance << 12 | staged row << 6 | column are unique and
+// order ties by raster index, so a distance costs the top two two minima and a maximum.
+// The logic pipe (16 XORs, the carry-save adders, addresses, the top two) and the
+// population-count pipe (12 counts) bound it about equally; packed keys and the staged
+// order take several of the logic pipe's operations per distance away.  Measured (GB300; before:
+// rotated chunks, compares and selects): 640x480 at radius 2 / 8 / 16 34.4 -> 30.4, 301.6 ->
+// 255.3 and 1,790 -> 1,423 us, 1920x1080 at radius 8 1,906 -> 1,611 us, 97x70 at radius 8
+// 67.5 -> 54.1 us, radius 0 unchanged.  Two pixels per thread (a candidate's loads serve
+// both) took 275 us at 640x480, radius 8: too few warps; copies by cp.async lose 18% at
+// radius 0.
 __global__ void __launch_bounds__(kMatchThreads) dense_match_kernel(const uint4* __restrict__ da,
                                                                     const uint4* __restrict__ db, int width,
                                                                     int height, int radius, int k, int r_milli,
                                                                     latch_match* __restrict__ out) {
     extern __shared__ uint4 s_desc[];
-    const int side = kMTile + 2 * radius;
+    const int side = kMTile + 2 * radius, cells = side * side;
     const int x0 = blockIdx.x * kMTile, y0 = blockIdx.y * kMTile;
     griddep_wait();
     griddep_launch_dependents();
-    for (int i = threadIdx.x; i < side * side * 4; i += kMatchThreads) {
-        const int cell = i >> 2, q = i & 3;
+    for (int i = threadIdx.x; i < (cells + 7) / 8 * 32; i += kMatchThreads) {
+        const int cell = (i >> 5) * 8 + (i & 7), q = (i >> 3) & 3;
         const int ry = cell / side, rx = cell - ry * side;
         const int gy = y0 - radius + ry, gx = x0 - radius + rx;
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (gx >= 0 && gx < width && gy >= 0 && gy < height) v = db[(static_cast<int64_t>(gy) * width + gx) * 4 + q];
-        s_desc[chunk_slot(cell, q)] = v;
+        if (cell < cells && gx >= 0 && gx < width && gy >= 0 && gy < height)
+            s_desc[i] = db[(static_cast<int64_t>(gy) * width + gx) * 4 + q];
     }
     const int tx = threadIdx.x % kMTile, ty = threadIdx.x / kMTile;
     const int px = x0 + tx, py = y0 + ty;
@@ -204,42 +218,38 @@ __global__ void __launch_bounds__(kMatchThreads) dense_match_kernel(const uint4*
             const uint4 v = src[q];
             a[4 * q] = v.x, a[4 * q + 1] = v.y, a[4 * q + 2] = v.z, a[4 * q + 3] = v.w;
         }
-    } else {
-#pragma unroll
-        for (int w = 0; w < 16; ++w) a[w] = 0;
     }
     __syncthreads();
     if (!live) return;
-    int d1 = 0x7fffffff, d2 = 0x7fffffff, i1 = -1, i2 = -1;
-    const int ylo = py - radius < 0 ? 0 : py - radius, yhi = py + radius >= height ? height - 1 : py + radius;
-    const int xlo = px - radius < 0 ? 0 : px - radius, xhi = px + radius >= width ? width - 1 : px + radius;
-    for (int qy = ylo; qy <= yhi; ++qy) {
-        const int rowcell = (qy - y0 + radius) * side - x0 + radius;
-        for (int qx = xlo; qx <= xhi; ++qx) {
-            const int cell = rowcell + qx;
+    uint32_t m1 = kNoKey, m2 = kNoKey;
+    // staged rows and columns of the candidates inside B
+    const int rx_lo = max(tx, radius - x0), rx_hi = min(tx + 2 * radius, width - 1 - x0 + radius);
+    const int ry_lo = max(ty, radius - y0), ry_hi = min(ty + 2 * radius, height - 1 - y0 + radius);
+    for (int ry = ry_lo; ry <= ry_hi; ++ry) {
+        for (int rx = rx_lo; rx <= rx_hi; ++rx) {
+            const uint4* c = staged_cell(s_desc, ry * side + rx);
             uint32_t x[16];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const uint4 v = s_desc[chunk_slot(cell, q)];
+                const uint4 v = c[8 * q];
                 x[4 * q] = v.x ^ a[4 * q], x[4 * q + 1] = v.y ^ a[4 * q + 1];
                 x[4 * q + 2] = v.z ^ a[4 * q + 2], x[4 * q + 3] = v.w ^ a[4 * q + 3];
             }
-            const int d = popc16(x);
-            const int idx = qy * width + qx;
-            if (d < d1) {
-                d2 = d1, i2 = i1;
-                d1 = d, i1 = idx;
-            } else if (d < d2) {
-                d2 = d, i2 = idx;
-            }
+            const uint32_t key = (static_cast<uint32_t>(popc16(x)) << kOrdBits) + static_cast<uint32_t>(ry << 6 | rx);
+            m2 = min(m2, max(m1, key));
+            m1 = min(m1, key);
         }
     }
+    auto index = [&](uint32_t key) {
+        const int ry = key >> 6 & 63, rx = key & 63;
+        return (y0 - radius + ry) * width + x0 - radius + rx;
+    };
     latch_match m;
-    m.idx1 = i1;
-    m.dist1 = static_cast<uint16_t>(d1);
-    const bool has2 = k == 2 && i2 >= 0;
-    m.idx2 = has2 ? i2 : -1;
-    m.dist2 = has2 ? static_cast<uint16_t>(d2) : 0xffff;
+    m.idx1 = index(m1);  // the pixel itself is always a candidate
+    m.dist1 = static_cast<uint16_t>(m1 >> kOrdBits);
+    const bool has2 = k == 2 && m2 != kNoKey;
+    m.idx2 = has2 ? index(m2) : -1;
+    m.dist2 = has2 ? static_cast<uint16_t>(m2 >> kOrdBits) : 0xffff;
     if (k == 1)
         m.accepted = 1;
     else
@@ -252,7 +262,7 @@ __global__ void __launch_bounds__(kMatchThreads) dense_match_kernel(const uint4*
 
 static size_t dense_match_smem_bytes(int radius) {
     const size_t side = static_cast<size_t>(kMTile + 2 * radius);
-    return side * side * kDescBytes;
+    return (side * side + 7) / 8 * 8 * kDescBytes;  // whole groups of eight cells
 }
 
 cudaError_t launch_dense_extract(const latch_context* ctx, const latch_image* img, uint8_t* d_out,
