@@ -4,8 +4,8 @@
 // descriptors (32 words in registers); a block streams its slice of the train set
 // through shared memory in double-buffered tiles (cp.async) and every thread computes
 // the exact Hamming distance of its queries to every train descriptor of the slice.
-// Half of the 16 XOR words of a pair are folded by a carry-save adder tree into words
-// of weight 1, 2, 4 and 8 (4 population counts for 8), the other half are counted
+// Eleven of the 16 XOR words of a pair are folded by a carry-save adder tree into words
+// of weight 1, 2, 4 and 8 (4 population counts for 11), the others are counted
 // directly, which balances the logic pipe against the population-count pipe.  Keys are
 // (distance << 21 | index in the slice), unique within a slice, so min / second-min
 // is the top-2 with ties to the lowest index.  With one slice the block writes the
