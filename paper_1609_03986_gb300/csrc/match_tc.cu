@@ -57,7 +57,8 @@
 // left above 720 clocks is the accumulators' round trip (MMA end, commit, TMEM loads of 20
 // warps, arrivals of both blocks, next MMA: about 1,200 clocks for two accumulators in
 // flight); three accumulators of 160 columns are slower (2,357 us: the epilogue's time per
-// unit hardly depends on its columns).
+// unit hardly depends on its columns).  Short walks are bound by the top-two updates of
+// their first units instead; there the pairs of a tile exchange row bounds (single problems).
 #include <cuda.h>
 
 #include <cmath>
@@ -98,6 +99,10 @@ constexpr uint32_t kSfbCol = kSfaCol + 8;  // scale factors of B: 4 columns per 
 constexpr uint32_t kScaleOne = 0x7F7F7F7Fu;  // four UE8M0 scale factors 2^0 (columns 496-511 all hold it)
 constexpr uint32_t kIdesc64 = idesc_mxf4_e2m1(kRowsQ, kColsB);
 constexpr uint32_t kIdesc96 = kIdesc64 | kIdescK96;
+// A walk exchanges its row bounds with the tile's other pairs over its first units; beyond,
+// updates are rare and the exchange costs more than it saves (16,384 x 1,048,576: 2,019 us
+// when every unit does it).
+constexpr int32_t kShareUnits = 64;
 constexpr int32_t kNoBound = 1024;      // a distance bound above every distance (512 bits)
 constexpr int64_t kFusedUnitsPerPair = 64;  // longer launches combine the tiles' records in a separate pass
 constexpr int64_t kWholeTilesPerPair = 8;   // batches with this many query tiles per pair share whole tiles
@@ -334,12 +339,16 @@ __device__ __forceinline__ latch_match final_match(uint64_t k1, uint64_t k2, int
 
 // tile_cnt: per-query-tile arrival counters, zero at launch and zero again after a
 // complete launch; NULL = leave the combination to match_merge_kernel.
+// row_bounds (single problems): per query row the distance bound the pairs that share its
+// tile have reached, as kNoBound - bound (0: none yet), zero at launch; NULL = each pair's
+// own bounds only.
 template <int NP>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_constant__ CUtensorMap tmq,
                                                               const __grid_constant__ CUtensorMap tmt,
                                                               const __grid_constant__ MatchBatchT<NP> batch,
                                                               uint64_t* __restrict__ partials,
                                                               int32_t* __restrict__ tile_cnt,
+                                                              int32_t* __restrict__ row_bounds,
                                                               latch_match* __restrict__ out,
                                                               uint32_t* __restrict__ flags) {
     extern __shared__ uint8_t smem_raw[];
@@ -609,6 +618,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) match_t
                 }
             };
             const int32_t n_end = u.n + run.len;
+            // The first units of a walk are its dearest: as long as a row has met few columns
+            // some row of nearly every warp takes an update.  The pairs that walk other parts
+            // of the same tile tighten the row's bound together: column group 0 takes the
+            // bound loaded a unit ago, publishes a lower one and loads again.  It is a bound
+            // like the block's own (two keys at that distance are in some pair's record), so
+            // the columns it excludes are in no final top two.
+            int32_t seen = 0;
+            const int32_t n_share = NP == 1 && row_bounds != nullptr && cg == 0 ? u.n + kShareUnits : u.n;
+            const int32_t grow = static_cast<int32_t>(u.m) * kRowsQ + row_in_tile;
             for (int32_t n = u.n; n < n_end; ++n) {
                 // after a failed wait a warp keeps walking the units without work, so that
                 // every warp reaches the barriers at the ends of query tiles
@@ -616,6 +634,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) match_t
                 if (!aborted) {
                     acc_par ^= 1u << acc;
                     tc_fence_after();
+                    if (NP == 1 && n < n_share) {
+                        const int32_t own = kNoBound - *static_cast<volatile int32_t*>(&sBound[row_in_block]);
+                        if (seen > own) atomicMin(&sBound[row_in_block], kNoBound - seen);
+                        if (own > seen) atomicMax(&row_bounds[grow], own);
+                        seen = *static_cast<volatile int32_t*>(&row_bounds[grow]);
+                    }
                     // the thread's columns (512 - 2 Hamming, exact integers) and the largest
                     // of each half in one round trip; the accumulator is free again as soon
                     // as they are in registers
@@ -751,16 +775,17 @@ __global__ void expand_kernel(const uint32_t* __restrict__ in, int64_t nwords, u
 }
 
 // The same for a single problem: the query set, then the train set behind it, and the
-// matcher's arrival counters cleared, in one launch.  (Two expansions and a memset in
+// matcher's arrival counters and row bounds cleared, in one launch.  (Two expansions and a memset in
 // front of the matcher cost about 2 us more: 10,000 x 10,000 descriptors match in 45
 // instead of 47 us.)
 __global__ void expand_two_kernel(const uint32_t* __restrict__ q, int64_t qwords, const uint32_t* __restrict__ t,
                                   int64_t twords, uint4* __restrict__ out, int32_t* __restrict__ counters,
-                                  int32_t ncounters) {
+                                  int32_t ncounters, int32_t* __restrict__ bounds, int32_t nbounds) {
     griddep_wait();
     griddep_launch_dependents();
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i < ncounters) counters[i] = 0;
+    if (i < nbounds) bounds[i] = 0;
     if (i < qwords)
         out[i] = expand_word_e2m1(q[i]);
     else if (i < qwords + twords)
@@ -889,8 +914,8 @@ static cudaError_t set_match_attributes() {
 
 template <int NP>
 static cudaError_t launch_match_np(const MatchBatch& full, const CUtensorMap& mapq, const CUtensorMap& mapt,
-                                   uint64_t* partials, int32_t* tile_cnt, latch_match* out, uint32_t* flags,
-                                   cudaStream_t stream) {
+                                   uint64_t* partials, int32_t* tile_cnt, int32_t* row_bounds, latch_match* out,
+                                   uint32_t* flags, cudaStream_t stream) {
     static unsigned long long attr_done = 0;
     {
         const cudaError_t e = once_per_device(&attr_done, set_match_attributes<NP>);
@@ -902,7 +927,7 @@ static cudaError_t launch_match_np(const MatchBatch& full, const CUtensorMap& ma
     cudaError_t e = cudaSuccess;
     if (b->units > 0)
         e = launch_chained(match_tc_kernel<NP>, dim3(static_cast<unsigned>(2 * b->grid)), dim3(kThreads), kSmemBytes,
-                           stream, mapq, mapt, *b, partials, tile_cnt, out, flags);
+                           stream, mapq, mapt, *b, partials, tile_cnt, row_bounds, out, flags);
     if (e == cudaSuccess && !tile_cnt && !b->whole_tiles && b->queries > 0) {
         const int threads = 256;
         const int64_t grid = (b->queries + threads - 1) / threads;
@@ -913,13 +938,14 @@ static cudaError_t launch_match_np(const MatchBatch& full, const CUtensorMap& ma
     return e;
 }
 
-cudaError_t launch_match_tc_rows(const MatchBatch& b, const uint8_t* exp, int64_t rows, uint64_t* partials, int32_t* tile_cnt, latch_match* out, uint32_t* flags,
-                                 cudaStream_t stream) {
+static cudaError_t launch_match_tc_bounds(const MatchBatch& b, const uint8_t* exp, int64_t rows, uint64_t* partials,
+                                          int32_t* tile_cnt, int32_t* row_bounds, latch_match* out, uint32_t* flags,
+                                          cudaStream_t stream) {
     if (b.queries == 0) return cudaSuccess;
     CUtensorMap mapq, mapt;
     if (b.units > 0 && !(make_map(&mapq, exp, rows, kRowsA) && make_map(&mapt, exp, rows, kRowsB)))
         return cudaErrorInvalidValue;
-    // a short launch (at most kFusedUnitsPerPair units per block) combines each query
+    // a short launch (at most kFusedUnitsPerPair units per pair) combines each query
     // tile's records itself, which saves the merge launch; a long one leaves them to
     // match_merge_kernel, because the combine at a tile's end (a fence and an atomic
     // round trip per block) holds the epilogue while the MMAs can run only an
@@ -929,9 +955,14 @@ cudaError_t launch_match_tc_rows(const MatchBatch& b, const uint8_t* exp, int64_
     for (int i = 0; i < b.count; ++i)
         if (b.p[i].nq > 0 && b.p[i].ntl == 0) fused = false;
     if (!fused) tile_cnt = nullptr;
-    if (b.count <= 1) return launch_match_np<1>(b, mapq, mapt, partials, tile_cnt, out, flags, stream);
-    if (b.count <= 16) return launch_match_np<16>(b, mapq, mapt, partials, tile_cnt, out, flags, stream);
-    return launch_match_np<kMaxProblems>(b, mapq, mapt, partials, tile_cnt, out, flags, stream);
+    if (b.count <= 1) return launch_match_np<1>(b, mapq, mapt, partials, tile_cnt, row_bounds, out, flags, stream);
+    if (b.count <= 16) return launch_match_np<16>(b, mapq, mapt, partials, tile_cnt, nullptr, out, flags, stream);
+    return launch_match_np<kMaxProblems>(b, mapq, mapt, partials, tile_cnt, nullptr, out, flags, stream);
+}
+
+cudaError_t launch_match_tc_rows(const MatchBatch& b, const uint8_t* exp, int64_t rows, uint64_t* partials,
+                                 int32_t* tile_cnt, latch_match* out, uint32_t* flags, cudaStream_t stream) {
+    return launch_match_tc_bounds(b, exp, rows, partials, tile_cnt, nullptr, out, flags, stream);
 }
 
 // Scratch: expanded rows (rows x kExpRowBytes), arrival counters, partial records.
@@ -964,28 +995,54 @@ size_t match_tc_scratch_bytes_sms(int64_t sms, int64_t nq, int64_t nt) {
     return r;
 }
 
+// Row bounds of a single problem (shared by the pairs of a tile), behind its scratch.
+static size_t row_bound_bytes(int64_t nq) { return static_cast<size_t>((nq + kRowsQ - 1) / kRowsQ) * kRowsQ * 4; }
+
 size_t match_tc_scratch_bytes(const latch_context* ctx, int64_t nq, int64_t nt) {
-    return match_tc_scratch_bytes_sms(ctx->sm_count, nq, nt);
+    return align_up(match_tc_scratch_bytes_sms(ctx->sm_count, nq, nt), 256) + row_bound_bytes(nq);
 }
 
-cudaError_t launch_match_tc(const latch_context* ctx, const uint8_t* q, int32_t nq, const uint8_t* t, int32_t nt,
-                            int32_t k, int32_t r_milli, latch_match* out, void* scratch, cudaStream_t stream) {
+// `bounds`: the scratch has row_bound_bytes(nq) more, 256-byte aligned behind the rest.
+static cudaError_t launch_match_single(const latch_context* ctx, const uint8_t* q, int32_t nq, const uint8_t* t,
+                                       int32_t nt, int32_t k, int32_t r_milli, latch_match* out, void* scratch,
+                                       bool bounds, cudaStream_t stream) {
     MatchBatch* b = new MatchBatch;
     single_problem(b, nq, nt, ctx->sm_count, k, r_milli);
     uint8_t* base = static_cast<uint8_t*>(scratch);
+    int32_t* cnt = match_tc_batch_counters(scratch, static_cast<int64_t>(nq) + nt);
+    // only pairs that share a tile have bounds to exchange.  Without / with the exchange, us per
+    // call: 2,340 x 60,000 58.6 / 53.2, 2,340 x 230,000 129.9 / 115.4, 5,000 x 230,000 195.0 /
+    // 183.6, 10,000 x 60,000 121.5 / 118.8
+    bounds = bounds && !b->whole_tiles && b->grid > b->tiles;
+    int32_t* row_bounds =
+        bounds ? reinterpret_cast<int32_t*>(
+                     base + align_up(match_tc_scratch_bytes_sms(ctx->sm_count, nq, nt), 256))
+               : nullptr;
     cudaError_t e = cudaSuccess;
     if (b->units > 0) {
         const int64_t qwords = static_cast<int64_t>(nq) * kDescWords, twords = static_cast<int64_t>(nt) * kDescWords;
         const int32_t ncounters = 2 * b->tiles;  // fewer than the query words
+        const int32_t nbounds = bounds ? b->tiles * kRowsQ : 0;
         const int threads = 256;
-        e = launch_chained(expand_two_kernel, dim3(static_cast<unsigned>((qwords + twords + threads - 1) / threads)),
+        const int64_t work = qwords + twords > nbounds ? qwords + twords : nbounds;
+        e = launch_chained(expand_two_kernel, dim3(static_cast<unsigned>((work + threads - 1) / threads)),
                            dim3(threads), 0, stream, reinterpret_cast<const uint32_t*>(q), qwords,
-                           reinterpret_cast<const uint32_t*>(t), twords, reinterpret_cast<uint4*>(base),
-                           match_tc_batch_counters(scratch, static_cast<int64_t>(nq) + nt), ncounters);
+                           reinterpret_cast<const uint32_t*>(t), twords, reinterpret_cast<uint4*>(base), cnt, ncounters,
+                           row_bounds, nbounds);
     }
-    if (e == cudaSuccess) e = launch_match_tc_batch(*b, nq + nt, b->tiles, scratch, out, ctx->d_flags, stream);
+    if (e == cudaSuccess) {
+        const size_t exp_bytes = align_up((static_cast<size_t>(nq) + nt) * kKBytes, 1024);
+        uint64_t* partials = reinterpret_cast<uint64_t*>(base + exp_bytes + match_tc_counter_bytes(b->tiles));
+        e = launch_match_tc_bounds(*b, base, static_cast<int64_t>(nq) + nt, partials, cnt, row_bounds, out, ctx->d_flags,
+                                   stream);
+    }
     delete b;
     return e;
+}
+
+cudaError_t launch_match_tc(const latch_context* ctx, const uint8_t* q, int32_t nq, const uint8_t* t, int32_t nt,
+                            int32_t k, int32_t r_milli, latch_match* out, void* scratch, cudaStream_t stream) {
+    return launch_match_single(ctx, q, nq, t, nt, k, r_milli, out, scratch, true, stream);
 }
 
 }  // namespace latch
@@ -1076,7 +1133,8 @@ extern "C" latch_status hamming_match_noalloc(const uint8_t* d_query, int32_t nq
     shim.sm_count = sms;
     shim.d_flags = flags;
     const int32_t r_milli = static_cast<int32_t>(std::round(static_cast<double>(ratio) * 1000.0));
-    e = launch_match_tc(&shim, d_query, nq, d_train, nt, k, r_milli, d_out, bytes + kStaticFlagBytes, cs);
+    const bool bounds = (need + 255) / 256 * 256 + row_bound_bytes(nq) <= kStaticScratchBytes;  // left out where they do not fit
+    e = launch_match_single(&shim, d_query, nq, d_train, nt, k, r_milli, d_out, bytes + kStaticFlagBytes, bounds, cs);
     if (e != cudaSuccess) return fail(nullptr, LATCH_ECUDA, "tensor match launch: %s", cudaGetErrorString(e));
     return LATCH_OK;
 }
