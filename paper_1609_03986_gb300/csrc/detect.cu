@@ -38,7 +38,7 @@ namespace {
 
 using namespace sm103;
 
-constexpr int kCellD = 32;          // detection cell (the extraction's cell size)
+constexpr int kCellD = 32;          // detection cell
 constexpr int kHaloD = 16;          // staged halo: the centroid disc (15) + 1
 constexpr int kTileD = kCellD + 2 * kHaloD;  // 64
 constexpr int kApron = kCellD + 2;           // scores of the cell and a 1-pixel apron

@@ -19,7 +19,8 @@ Ceilings:
   tensor       4-bit float (E2M1): the measured dense bf16 GEMM throughput
                x 6 (the nominal dense fp4 / bf16 ratio), burst for a kernel timed
                alone and sustained for one timed inside a long step; beside it the
-               measured issue rate of the block-scaled E2M1 MMA (4x bf16 per clock).
+               measured issue rate of the matcher's own MMA sequence (K = 96, 96 and 64
+               of each 256 values, two SMs per MMA: 5.33x bf16 per clock).
 Per-clock pipe rates come from a throughput probe on this GPU, stored in
 ``pipe_rates.json``; the clocks and the bf16 / HBM figures from the driver's
 measured-peaks file.
@@ -172,8 +173,9 @@ def detection(ms: float, pixels: int, workload: str, peaks_path: str):
 def tensor_match(ms: float, pairs: float, workload: str, peaks_path: str, sustained: bool):
     """Tensor matcher: 1,024 flop per pair on the block-scaled E2M1 MMA.  `peak` is
     the measured bf16 GEMM x 6, the nominal dense fp4 / bf16 ratio (13.5 / 2.25
-    PFLOP/s); `issue_view` compares with the measured issue rate of the MMA form the
-    kernel uses (kind::mxf4, one CTA per MMA), 4x the bf16 rate per clock."""
+    PFLOP/s); `issue_view` compares with the measured issue rate of the MMA sequence the
+    kernel uses (kind::mxf4, CTA pairs, 6 MMAs per 512 values), 5.33x the bf16 rate per
+    clock."""
     peaks, pk = _peaks(peaks_path)
     rates, rk = pipe_rates()
     bf16 = float(peaks["bf16_tflops_sustained" if sustained else "bf16_tflops"])
@@ -182,11 +184,11 @@ def tensor_match(ms: float, pairs: float, workload: str, peaks_path: str, sustai
          "achieved": achieved, "peak": 6.0 * bf16,
          "traffic": traffic("match_tc", "match_tc.cu", workload)}
     pr = rates["per_sm_per_clock"]
-    if "mma_mxf4_flop" in pr and "mma_bf16_flop" in pr:
-        ratio = pr["mma_mxf4_flop"] / pr["mma_bf16_flop"]
+    if "mma_mxf4_pair_k512_flop" in pr and "mma_bf16_flop" in pr:
+        ratio = pr["mma_mxf4_pair_k512_flop"] / pr["mma_bf16_flop"]
         r["issue_view"] = {"peak": ratio * bf16, "frac": achieved / (ratio * bf16),
                            "peak_model": f"bf16 {'sustained' if sustained else 'burst'} x {ratio:.2f}, the measured "
-                                         "kind::mxf4 / kind::f16 issue ratio"}
+                                         "issue ratio of the pair kind::mxf4 sequence to kind::f16"}
     return _finish(r, f"{pk} bf16 {'sustained' if sustained else 'burst'} x 6 (nominal fp4/bf16)")
 
 
