@@ -101,7 +101,7 @@ constexpr uint32_t kIdesc64 = idesc_mxf4_e2m1(kRowsQ, kColsB);
 constexpr uint32_t kIdesc96 = kIdesc64 | kIdescK96;
 // A walk exchanges its row bounds with the tile's other pairs over its first units; beyond,
 // updates are rare and the exchange costs more than it saves (16,384 x 1,048,576: 2,019 us
-// when every unit does it).
+// when every unit of the walk does it, 1,755 with 64).
 constexpr int32_t kShareUnits = 64;
 constexpr int32_t kNoBound = 1024;      // a distance bound above every distance (512 bits)
 constexpr int64_t kFusedUnitsPerPair = 64;  // longer launches combine the tiles' records in a separate pass
@@ -342,7 +342,9 @@ __device__ __forceinline__ latch_match final_match(uint64_t k1, uint64_t k2, int
 // row_bounds (single problems): per query row the distance bound the pairs that share its
 // tile have reached, as kNoBound - bound (0: none yet), zero at launch; NULL = each pair's
 // own bounds only.
-template <int NP>
+// kShare: row_bounds is given (a kernel of its own: the exchange's registers slow long walks
+// by 3%).
+template <int NP, bool kShare>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) match_tc_kernel(const __grid_constant__ CUtensorMap tmq,
                                                               const __grid_constant__ CUtensorMap tmt,
                                                               const __grid_constant__ MatchBatchT<NP> batch,
@@ -625,7 +627,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) match_t
             // like the block's own (two keys at that distance are in some pair's record), so
             // the columns it excludes are in no final top two.
             int32_t seen = 0;
-            const int32_t n_share = NP == 1 && row_bounds != nullptr && cg == 0 ? u.n + kShareUnits : u.n;
+            const int32_t n_share = kShare && cg == 0 ? u.n + kShareUnits : u.n;
             const int32_t grow = static_cast<int32_t>(u.m) * kRowsQ + row_in_tile;
             for (int32_t n = u.n; n < n_end; ++n) {
                 // after a failed wait a warp keeps walking the units without work, so that
@@ -634,7 +636,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) match_t
                 if (!aborted) {
                     acc_par ^= 1u << acc;
                     tc_fence_after();
-                    if (NP == 1 && n < n_share) {
+                    if (kShare && n < n_share) {
                         const int32_t own = kNoBound - *static_cast<volatile int32_t*>(&sBound[row_in_block]);
                         if (seen > own) atomicMin(&sBound[row_in_block], kNoBound - seen);
                         if (own > seen) atomicMax(&row_bounds[grow], own);
@@ -909,7 +911,10 @@ static void shrink(const MatchBatch& b, MatchBatchT<NP>* o) {
 
 template <int NP>
 static cudaError_t set_match_attributes() {
-    return cudaFuncSetAttribute(match_tc_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    const cudaError_t e =
+        cudaFuncSetAttribute(match_tc_kernel<NP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e != cudaSuccess || NP > 1) return e;
+    return cudaFuncSetAttribute(match_tc_kernel<NP, NP == 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
 }
 
 template <int NP>
@@ -926,7 +931,7 @@ static cudaError_t launch_match_np(const MatchBatch& full, const CUtensorMap& ma
     shrink(full, b);
     cudaError_t e = cudaSuccess;
     if (b->units > 0)
-        e = launch_chained(match_tc_kernel<NP>, dim3(static_cast<unsigned>(2 * b->grid)), dim3(kThreads), kSmemBytes,
+        e = launch_chained(row_bounds ? match_tc_kernel<NP, NP == 1> : match_tc_kernel<NP, false>, dim3(static_cast<unsigned>(2 * b->grid)), dim3(kThreads), kSmemBytes,
                            stream, mapq, mapt, *b, partials, tile_cnt, row_bounds, out, flags);
     if (e == cudaSuccess && !tile_cnt && !b->whole_tiles && b->queries > 0) {
         const int threads = 256;
@@ -1010,10 +1015,12 @@ static cudaError_t launch_match_single(const latch_context* ctx, const uint8_t* 
     single_problem(b, nq, nt, ctx->sm_count, k, r_milli);
     uint8_t* base = static_cast<uint8_t*>(scratch);
     int32_t* cnt = match_tc_batch_counters(scratch, static_cast<int64_t>(nq) + nt);
-    // only pairs that share a tile have bounds to exchange.  Without / with the exchange, us per
-    // call: 2,340 x 60,000 58.6 / 53.2, 2,340 x 230,000 129.9 / 115.4, 5,000 x 230,000 195.0 /
-    // 183.6, 10,000 x 60,000 121.5 / 118.8
-    bounds = bounds && !b->whole_tiles && b->grid > b->tiles;
+    // only pairs that share a tile have bounds to exchange, and only short walks gain (up to
+    // about 500 units).  Without / with the exchange, us per call: 2,340 x 60,000 58.6 / 53.2,
+    // 2,340 x 230,000 129.9 / 115.4, 5,000 x 230,000 195.1 / 184.9, 10,000 x 60,000 121.9 /
+    // 117.9, 10,000 x 230,000 (500 units) 313.1 / 312.1; 10,000 x 1,048,576 1,128 / 1,156
+    // and, with 1.2 pairs per tile, 16,384 x 230,000 448 / 461
+    bounds = bounds && !b->whole_tiles && 2 * b->grid > 3 * b->tiles && b->units <= 512 * b->grid;
     int32_t* row_bounds =
         bounds ? reinterpret_cast<int32_t*>(
                      base + align_up(match_tc_scratch_bytes_sms(ctx->sm_count, nq, nt), 256))
