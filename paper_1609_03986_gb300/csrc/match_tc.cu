@@ -658,6 +658,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) match_t
                     const float vmin = fmaxf(
                         static_cast<float>(512 - 2 * *static_cast<volatile int32_t*>(&sBound[row_in_block])), vown2);
                     tmem_ld_wait();
+#pragma unroll
+                    for (int h = 0; h < kLds; ++h) tmem_arrived(v[h], mx[h]);
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive_cluster(acc_empty0 + 8u * static_cast<uint32_t>(acc));

@@ -292,6 +292,15 @@ __device__ __forceinline__ void tmem_ld_32x32b_x8(uint32_t taddr, uint32_t (&v)[
 
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
+// Directly after tmem_ld_wait(): ties the registers of a reducing load to it.  The wait
+// names no registers, so the compiler may move plain arithmetic on them above it.
+template <int N>
+__device__ __forceinline__ void tmem_arrived(uint32_t (&v)[N], float& mx) {
+#pragma unroll
+    for (int j = 0; j < N; ++j) asm volatile("" : "+r"(v[j]));
+    asm volatile("" : "+f"(mx));
+}
+
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of 128
 // bytes in 8-row groups 1024 bytes apart.  `addr` must lie in a 1024-byte aligned
 // tile (the k-offset inside the swizzle atom is added to the start address).
