@@ -59,6 +59,60 @@ __host__ __device__ __forceinline__ int64_t split_owner(int64_t u, int64_t units
     return c;
 }
 
+// A pair of blocks c of the G = b.grid walks the launch as shares: consecutive units of one
+// problem p from unit (m, n) on, `left` of them (p == count: there is none).
+struct Share {
+    int32_t p, m, n, cs;  // cs: the share's index in problem p (unit shares)
+    int64_t left;
+};
+
+// Unit shares: the first problem from p on in which pair c has a non-empty share, units
+// [start(c'), start(c' + 1)) of its U units with c' = (c - unit0) mod G (the rotation
+// continues each problem where the previous one ended, so problems smaller than G still
+// spread over all pairs).  All pairs thus work on the same problem at a time and share its
+// train set in L2.  A pair's record of tile g in problem p sits in slot g + c' + p (G - 1):
+// within a problem a later share never touches an earlier tile, and the problems' slot
+// ranges follow one another.  Out of line: it divides, and runs only where a share starts.
+template <class B>
+__host__ __device__ __noinline__ Share unit_share(const B& b, int p, int64_t c) {
+    for (; p < b.count; ++p) {
+        const MatchProblem& P = b.p[p];
+        const int64_t U = static_cast<int64_t>(P.mt) * P.ntl;
+        if (U == 0) continue;
+        const int64_t rot = P.unit0 % b.grid;
+        const int64_t cp = c >= rot ? c - rot : c - rot + b.grid;
+        const int64_t s0 = split_start(cp, U, b.grid), s1 = split_start(cp + 1, U, b.grid);
+        if (s1 > s0) {
+            const int32_t m = static_cast<int32_t>(s0 / P.ntl);
+            return Share{p, m, static_cast<int32_t>(s0 - static_cast<int64_t>(m) * P.ntl), static_cast<int32_t>(cp),
+                         s1 - s0};
+        }
+    }
+    return Share{b.count, 0, 0, 0, 0};
+}
+
+// Whole tiles: query tile g of the launch, in problem p or a later one.
+template <class B>
+__host__ __device__ __noinline__ Share tile_share(const B& b, int p, int64_t g) {
+    if (g >= b.tiles) return Share{b.count, 0, 0, 0, 0};
+    int lo = p, hi = b.count - 1;  // the first problem whose tiles end behind g
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (static_cast<int64_t>(b.p[mid].g0) + b.p[mid].mt > g) hi = mid; else lo = mid + 1;
+    }
+    return Share{lo, static_cast<int32_t>(g - b.p[lo].g0), 0, 0, b.p[lo].ntl};
+}
+
+// Pair c's first share, and the one after its share that ended in tile m of problem p.
+template <class B>
+__host__ __device__ __forceinline__ Share first_share(const B& b, int64_t c) {
+    return b.whole_tiles ? tile_share(b, 0, c) : unit_share(b, 0, c);
+}
+template <class B>
+__host__ __device__ __forceinline__ Share share_after(const B& b, int p, int32_t m, int64_t c) {
+    return b.whole_tiles ? tile_share(b, p, static_cast<int64_t>(b.p[p].g0) + m + b.grid) : unit_share(b, p + 1, c);
+}
+
 __device__ __forceinline__ void top2_insert_u64(uint64_t key, uint64_t& k1, uint64_t& k2) {
     const uint64_t hi = key > k1 ? key : k1;
     k1 = key < k1 ? key : k1;

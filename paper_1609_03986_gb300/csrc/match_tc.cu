@@ -14,8 +14,8 @@
 // boxes).  The blocks work in pairs (clusters of two on the two SMs of a TPC, one block
 // per SM, persistent); a pair's MMAs (cta_group::2, M = 256) take a tile of 256 queries,
 // 128 in each block, and 240 train rows, 120 in each block's shared memory.  The units
-// (problem, 256-query tile, 240-train tile) of all problems are linearised and split into
-// one contiguous range per pair:
+// (problem, 256-query tile, 240-train tile) of all problems are shared out over the pairs
+// (match_common.cuh); in a pair:
 //   warp 0     TMA producer of its block's half: the query rows (128 rows x 256 B, 32 KB)
 //              stay resident while consecutive units share them; train chunks (120 rows x
 //              128 B, half of K) go through a 12-stage ring, 128-byte swizzle; both
@@ -140,52 +140,6 @@ struct Smem {
 constexpr int kSmemBytes = Smem::total + 1024;
 static_assert(kSmemBytes <= 227 * 1024, "shared memory per block");
 
-// Walks the units of pair c: for every problem in turn, the pair's share of that
-// problem's U units, [start(c'), start(c' + 1)) with start(x) = floor(x U / G) and
-// c' = (c - unit0) mod G (the rotation continues each problem where the previous
-// one ended, so problems smaller than G still spread over all blocks), without
-// dividing inside a share.  All blocks thus work on the same problem at a time and
-// share its train set in L2.  last_of_tile(): the next unit of the walk is in
-// another query tile.  A block's record of tile g in problem p sits in slot
-// g + c' + p (G - 1): within a problem a later share never touches an earlier
-// tile, and the problems' slot ranges follow one another.
-// A block's share of one problem: the first unit (m, n), the share index and the
-// number of units; p == count when there is none left.
-struct Share {
-    int32_t p, m, n, cs;
-    int64_t left;
-};
-
-// The first problem from p on in which block c has a non-empty share.  Out of line:
-// it divides, and runs only where a share starts.
-template <class B>
-__device__ __noinline__ Share next_share(const B& b, int p, int64_t c) {
-    for (; p < b.count; ++p) {
-        const MatchProblem& P = b.p[p];
-        const int64_t U = static_cast<int64_t>(P.mt) * P.ntl;
-        if (U == 0) continue;
-        if (b.whole_tiles) {
-            // tiles [start(c'), start(c' + 1)) of the problem's mt, c' rotated by the
-            // problem's first tile index
-            const int64_t rot = P.g0 % b.grid;
-            const int64_t cp = c >= rot ? c - rot : c - rot + b.grid;
-            const int64_t t0 = split_start(cp, P.mt, b.grid), t1 = split_start(cp + 1, P.mt, b.grid);
-            if (t1 > t0)
-                return Share{p, static_cast<int32_t>(t0), 0, static_cast<int32_t>(cp), (t1 - t0) * P.ntl};
-            continue;
-        }
-        const int64_t rot = P.unit0 % b.grid;
-        const int64_t cp = c >= rot ? c - rot : c - rot + b.grid;
-        const int64_t s0 = split_start(cp, U, b.grid), s1 = split_start(cp + 1, U, b.grid);
-        if (s1 > s0) {
-            const int32_t m = static_cast<int32_t>(s0 / P.ntl);
-            return Share{p, m, static_cast<int32_t>(s0 - static_cast<int64_t>(m) * P.ntl), static_cast<int32_t>(cp),
-                         s1 - s0};
-        }
-    }
-    return Share{b.count, 0, 0, 0, 0};
-}
-
 // The fields of the current problem that the walk needs every unit are kept in
 // registers (reading the problem table, a kernel parameter, with a run-time index
 // costs hundreds of cycles per unit on the MMA warp's path).
@@ -200,8 +154,7 @@ struct UnitIter {
     int32_t nt;     // train rows of problem p
     int64_t left;   // units left in the share, the current one included
     template <class B>
-    __device__ __forceinline__ void take(const B& b, int from, int64_t c) {
-        const Share s = next_share(b, from, c);
+    __device__ __forceinline__ void set(const B& b, const Share& s) {
         p = s.p;
         m = s.m;
         n = s.n;
@@ -218,7 +171,7 @@ struct UnitIter {
     template <class B>
     __device__ __forceinline__ void init(const B& b, int64_t c) {
         count = b.count;
-        take(b, 0, c);
+        set(b, first_share(b, c));
     }
     template <class B>
     __device__ __forceinline__ bool done(const B&) const { return p >= count; }
@@ -233,7 +186,7 @@ struct UnitIter {
     template <class B>
     __device__ __forceinline__ void next(const B& b, int64_t c) {
         if (--left == 0) {
-            take(b, p + 1, c);
+            set(b, share_after(b, p, m, c));
             return;
         }
         if (++n == ntl) {
@@ -265,7 +218,7 @@ struct RunIter {
     template <class B>
     __device__ __forceinline__ void next(const B& b, int64_t c) {
         if (len == u.left) {
-            u.take(b, u.p + 1, c);  // the share ends with this run
+            u.set(b, share_after(b, u.p, u.m, c));  // the share ends with this run
         } else {
             u.left -= len;          // the run ends with its tile
             ++u.m;
@@ -282,10 +235,6 @@ struct RunIter {
 // so the owners are those of the tile's ntl units.
 template <class B, class F>
 __device__ __forceinline__ int64_t for_each_owner(const B& b, const MatchProblem& P, int64_t m, F&& f) {
-    if (b.whole_tiles) {
-        f(split_owner(m, P.mt, b.grid));
-        return 1;
-    }
     const int64_t U = static_cast<int64_t>(P.mt) * P.ntl;
     const int64_t u0 = m * P.ntl;
     if (U >= b.grid) {
@@ -300,7 +249,6 @@ __device__ __forceinline__ int64_t for_each_owner(const B& b, const MatchProblem
 // Number of blocks that hold a record of query tile m of problem P.
 template <class B>
 __device__ __forceinline__ int64_t tile_owner_count(const B& b, const MatchProblem& P, int64_t m) {
-    if (b.whole_tiles) return 1;
     const int64_t U = static_cast<int64_t>(P.mt) * P.ntl;
     if (U < b.grid) return P.ntl;
     const int64_t u0 = m * P.ntl;
@@ -860,10 +808,15 @@ void plan_match_batch(MatchBatch* b, int count, int64_t max_sms) {
     b->queries = queries;
     const int64_t pairs = max_sms / 2 > 0 ? max_sms / 2 : 1;
     b->grid = units < pairs ? units : pairs;
-    // whole query tiles per share when there are enough of them to balance the
-    // blocks (the block that walks a whole tile writes its matches directly, and a
-    // tile's walk pays its start-up -- the first units' top-two updates -- once);
-    // not when some problem has queries but no train rows (its tiles have no unit)
+    // whole query tiles dealt out to the pairs when there are enough of them to balance the
+    // pairs (the one that walks a whole tile writes its matches directly, and a tile's walk
+    // pays its start-up -- the first units' top-two updates -- once); not when some problem
+    // has queries but no train rows (its tiles have no unit).  Tile g goes to pair g mod G:
+    // cut into shares problem by problem, the few tiles of a problem fell on the same pairs
+    // again and again where their number and G have a common divisor (2 tiles and 76 pairs:
+    // on every second pair).  Matching of 1,128 image pairs on GB300, that way and this way:
+    // 300 descriptors an image 957 / 269 us, 1,000 1,388 / 833, 2,340 3,150 / 2,181, 5,000
+    // 7,507 / 7,014.
     bool whole = g >= kWholeTilesPerPair * b->grid;
     for (int i = 0; i < count; ++i)
         if (b->p[i].nq > 0 && b->p[i].ntl == 0) whole = false;
