@@ -15,8 +15,9 @@
 //                  third of it per warp, into a staging buffer, column of words by column
 //                  of words (word (cx, y) of the window at 48 cx + y);
 //   16 evaluators  first copy the batch's staged words into tensor memory, window j in
-//                  TMEM lane j of every lane quarter, which frees the staging buffer for
-//                  the next batch; then evaluate Eq. 1, all 32 lanes on the same triplet:
+//                  TMEM lane j of every lane quarter, and evaluate the triplets that no
+//                  quarter holds from the staged windows, which frees the staging buffer
+//                  for the next batch; then evaluate the others by Eq. 1, all 32 lanes on the same triplet:
 //                  a patch is two or three columns of words, so as many 8-row TMEM loads
 //                  bring it, its rows are aligned by funnel shifts, and D1 - D2 =
 //                  (sum C1^2 - sum C2^2) - 2 (sum A.C1 - sum A.C2) by __dp4a, all exact in
@@ -81,8 +82,6 @@ constexpr int kWarpBlocks = kBlocks / kGroupWarps;         // 6 per builder warp
 constexpr int kTmemCols = 512;
 constexpr int kTmLast = kTmemCols - 8;  // last column an 8-column load may start at
 constexpr int kStageWords = kWordCols * kWin + 1;          // odd: the 32 lanes' copies hit 32 banks
-constexpr int kExtRows = kWin - 42;     // the rows quarter 0 lacks, kept in shared memory too
-constexpr int kExtWords = kExtRows * kWordCols + 1;        // odd, as above
 constexpr int kOutWords = 33;           // descriptor word w of lane l at 33 w + l
 constexpr int kSlots = 8;               // tiles in flight at most, per producer
 constexpr int kClasses = 3;             // tile box sizes per launch
@@ -95,8 +94,9 @@ static_assert(kBuildWarps * kBuildRegs + 4 * kProducerRegs + kEvalWarps * kEvalR
 // `nc` columns of words from byte column `b0` on, rows r0 .. r0 + nr - 1, word (k, r) at
 // column k nr + r.  Each quarter lacks a different margin and starts at a different byte
 // of a word, and a triplet goes to a quarter that holds its three patches, of these to
-// one in which most of them start at a word (plan_triplets).  Quarter 0 takes those that
-// fit none, with rows 42..47 from shared memory.
+// one in which most of them start at a word (plan_triplets).  Those that fit none are
+// evaluated from the staged windows in shared memory, before these are given back, by the
+// warps of all quarters.
 struct Quarter {
     int32_t b0, nc, r0, nr;
 };
@@ -129,11 +129,13 @@ struct ExtractParams {
 // The triplets as the evaluators read them (from constant memory: the index is the
 // same for a whole warp, so the fields are unpacked once per warp), quarter by quarter
 // and class by class: a word per patch (anchor, companions), bits 0-4 the byte shift
-// times 8 (what a funnel shift takes), bits 16-24 the TMEM column of the patch's first
+// times 8 (what a funnel shift takes), bits 16-25 the TMEM column of the patch's first
 // word; bits 5-13 of the anchor's: the triplet's index.  A triplet's class has bit p set
-// when patch p does not start at a word (its rows must be aligned); class 8 (quarter 0):
-// it lies past the quarter's rows or three word columns from its first would not fit.
+// when patch p does not start at a word (its rows must be aligned); class 8 (kStaged): it
+// is read from the staged windows, its patches' first words being those of the window (word
+// (cx, y) at 48 cx + y), because the quarter does not hold it.
 constexpr int kTripClasses = 9;
+constexpr int kStaged = 8;
 struct LaneTriplets {
     uint32_t e[3][kBits];
     int16_t start[kQuarters][kTripClasses + 1];  // first entry of each class
@@ -208,7 +210,7 @@ struct LanesSmem {  // static part
     int abort;
 };
 
-constexpr size_t kFixedSmem = 128 + (static_cast<size_t>(kBatch) * kStageWords + 2 * kBatch * kExtWords) * 4;
+constexpr size_t kFixedSmem = 128 + static_cast<size_t>(kBatch) * kStageWords * 4;
 constexpr int kRingBytes = static_cast<int>((227 * 1024 - sizeof(LanesSmem) - kFixedSmem) / 128 * 128);
 constexpr size_t kDynSmem = kFixedSmem + kRingBytes;
 
@@ -246,25 +248,22 @@ __device__ __forceinline__ void align(uint32_t (&w)[3][8], uint32_t f) {
     }
 }
 
-// The rows that quarter 0 lacks, from `ext` (the lane's rows 42..47, 12 words each).  All
-// rows are loaded and the missing ones selected: a branch per row would cost a load's
-// latency each.
+// The patch whose first word is `f`, aligned, from a staged window: two word columns, and a
+// third where the patch reaches into it.
 template <int kRows>
-__device__ __forceinline__ void fill(uint32_t (&w)[3][8], uint32_t f, const uint32_t* ext) {
-    constexpr int nr = quarter_of(0).nr;
-    const int col = static_cast<int>(f >> 16), cx = col / nr, y0 = col - cx * nr;
-    if (y0 + kRows <= nr) return;
-    const uint32_t* x = ext + cx;
-    const int third = cx + 2 < kWordCols ? 2 : 1;
+__device__ __forceinline__ void load_staged(uint32_t (&w)[3][8], uint32_t f, const uint32_t* window) {
+    const uint32_t* x = window + (f >> 16);
 #pragma unroll
-    for (int r = 1; r < kRows; ++r) {
-        const int row = y0 + r - nr;
-        const uint32_t* xr = x + max(row, 0) * kWordCols;
-        const uint32_t v0 = xr[0], v1 = xr[1], v2 = xr[third];
-        w[0][r] = row >= 0 ? v0 : w[0][r];
-        w[1][r] = row >= 0 ? v1 : w[1][r];
-        w[2][r] = row >= 0 ? v2 : w[2][r];
+    for (int r = 0; r < kRows; ++r) {
+        w[0][r] = x[r];
+        w[1][r] = x[kWin + r];
+        w[2][r] = 0;
     }
+    if ((f & 31u) > 64 - 8 * kRows) {
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) w[2][r] = x[2 * kWin + r];
+    }
+    align<kRows>(w, f);
 }
 
 // The words of one triplet (LaneTriplets).
@@ -335,55 +334,11 @@ __device__ __forceinline__ void eval_class(const LaneTriplets& tt, int lo, int h
     tmem_ld_wait();
 }
 
-// Eq. 1 for one triplet of any class (kExt: class 8), not pipelined.
-template <bool kExt>
-__device__ __forceinline__ bool eval_any(const Words& f, uint32_t tm, uint32_t nr, const uint32_t* ext) {
-    uint32_t a[3][8], c[3][8], d[3][8];
-    request<true, true>(a, f.a, tm, nr);
-    request<true, true>(c, f.c1, tm, nr);
-    tmem_ld_wait();
-    arrive<true, 7>(a);
-    arrive<true, 7>(c);
-    request<true, true>(d, f.c2, tm, nr);
-    if constexpr (kExt) {
-        fill<7>(a, f.a, ext);
-        fill<7>(c, f.c1, ext);
-    }
-    align<7>(a, f.a);
-    align<7>(c, f.c1);
-    uint32_t ac1, cc1, ac2, cc2;
-    dot7(a, c, ac1, cc1);
-    tmem_ld_wait();
-    arrive<true, 7>(d);
-    if constexpr (kExt) fill<7>(d, f.c2, ext);
-    align<7>(d, f.c2);
-    dot7(a, d, ac2, cc2);
-    return farther(ac1, cc1, ac2, cc2);
-}
-
 // Eq. 1 with weighted 8x8 patches (Sec. 3.2, weighing pixels in LATCH patches):
 // D1 - D2 = sum w (C1 - C2)(C1 + C2 - 2 A), exact in int32 (|w (C1 - C2)(C1 + C2 - 2 A)|
 // <= 255 * 255^2 per pixel, 64 pixels).
-template <bool kExt>
-__device__ __forceinline__ bool eval_triplet_weighted(const Words& f, uint32_t tm, uint32_t nr, const uint32_t* ext,
-                                                      const PatchWeights& pw) {
-    uint32_t a[3][8], c[3][8], d[3][8];
-    request<true, true>(a, f.a, tm, nr);
-    request<true, true>(c, f.c1, tm, nr);
-    tmem_ld_wait();
-    arrive<true, 8>(a);
-    arrive<true, 8>(c);
-    if constexpr (kExt) {
-        fill<8>(a, f.a, ext);
-        fill<8>(c, f.c1, ext);
-    }
-    align<8>(a, f.a);
-    align<8>(c, f.c1);
-    request<true, true>(d, f.c2, tm, nr);
-    tmem_ld_wait();
-    arrive<true, 8>(d);
-    if constexpr (kExt) fill<8>(d, f.c2, ext);
-    align<8>(d, f.c2);
+__device__ __forceinline__ bool farther_weighted(const uint32_t (&a)[3][8], const uint32_t (&c)[3][8],
+                                                 const uint32_t (&d)[3][8], const PatchWeights& pw) {
     int acc = 0;
 #pragma unroll
     for (int r = 0; r < 8; ++r)
@@ -398,11 +353,56 @@ __device__ __forceinline__ bool eval_triplet_weighted(const Words& f, uint32_t t
     return acc > 0;
 }
 
-// The quarter's triplets [t0, t1) one at a time: weighted patches, a part of the chunks,
-// and class 8.
+// Eq. 1 for one triplet of any class of the quarter, not pipelined.
 template <bool kWeighted>
-__device__ __forceinline__ void eval_entries(const LaneTriplets& tt, const PatchWeights& pw, int lo, int hi, int ext0,
-                                             int mine, int t0, int t1, uint32_t tm, uint32_t nr, const uint32_t* ext,
+__device__ __forceinline__ bool eval_held(const Words& f, uint32_t tm, uint32_t nr, const PatchWeights& pw) {
+    constexpr int kRows = kWeighted ? 8 : 7;
+    uint32_t a[3][8], c[3][8], d[3][8];
+    request<true, true>(a, f.a, tm, nr);
+    request<true, true>(c, f.c1, tm, nr);
+    tmem_ld_wait();
+    arrive<true, kRows>(a);
+    arrive<true, kRows>(c);
+    if constexpr (!kWeighted) request<true, true>(d, f.c2, tm, nr);
+    align<kRows>(a, f.a);
+    align<kRows>(c, f.c1);
+    if constexpr (kWeighted) request<true, true>(d, f.c2, tm, nr);
+    uint32_t ac1 = 0, cc1 = 0, ac2, cc2;
+    if constexpr (!kWeighted) dot7(a, c, ac1, cc1);
+    tmem_ld_wait();
+    arrive<true, kRows>(d);
+    align<kRows>(d, f.c2);
+    if constexpr (kWeighted) return farther_weighted(a, c, d, pw);
+    dot7(a, d, ac2, cc2);
+    return farther(ac1, cc1, ac2, cc2);
+}
+
+// The same from the lane's staged window.  Its 42 to 63 shared-memory loads per triplet
+// (128 bytes per clock per SM, for all four quarters) and its instructions take about equally
+// long, some 250 clocks, and the builders wait for it: it serves the triplets that fit no
+// quarter, about 40 of 512 of a random table.  It is what bounds tables of far-apart patches:
+// 10,000 keypoints, every triplet across the window's diagonal, 72 us (the seeded table 51).
+// Before, quarter 0 alone evaluated them, its missing rows selected from shared memory: 218
+// and 53 us.
+template <bool kWeighted>
+__device__ __forceinline__ bool eval_staged(const Words& f, const uint32_t* window, const PatchWeights& pw) {
+    constexpr int kRows = kWeighted ? 8 : 7;
+    uint32_t a[3][8], c[3][8], d[3][8];
+    load_staged<kRows>(a, f.a, window);
+    load_staged<kRows>(c, f.c1, window);
+    load_staged<kRows>(d, f.c2, window);
+    if constexpr (kWeighted) return farther_weighted(a, c, d, pw);
+    uint32_t ac1, cc1, ac2, cc2;
+    dot7(a, c, ac1, cc1);
+    dot7(a, d, ac2, cc2);
+    return farther(ac1, cc1, ac2, cc2);
+}
+
+// Every fourth of the list entries [lo, hi) whose triplets lie in [t0, t1), one at a time:
+// weighted patches, a part of the chunks, and (kFromStage) the staged class.
+template <bool kWeighted, bool kFromStage>
+__device__ __forceinline__ void eval_entries(const LaneTriplets& tt, const PatchWeights& pw, int lo, int hi, int mine,
+                                             int t0, int t1, uint32_t tm, uint32_t nr, const uint32_t* window,
                                              uint32_t* bits, int lane) {
 #pragma unroll 1
     for (int p = lo + ((mine - lo) & 3); p < hi; p += 4) {
@@ -410,29 +410,20 @@ __device__ __forceinline__ void eval_entries(const LaneTriplets& tt, const Patch
         const int t = f.index();
         if (t < t0 || t >= t1) continue;
         bool bit;
-        if (p < ext0) {
-            if constexpr (kWeighted)
-                bit = eval_triplet_weighted<false>(f, tm, nr, ext, pw);
-            else
-                bit = eval_any<false>(f, tm, nr, ext);
-        } else {
-            if constexpr (kWeighted)
-                bit = eval_triplet_weighted<true>(f, tm, nr, ext, pw);
-            else
-                bit = eval_any<true>(f, tm, nr, ext);
-        }
+        if constexpr (kFromStage)
+            bit = eval_staged<kWeighted>(f, window, pw);
+        else
+            bit = eval_held<kWeighted>(f, tm, nr, pw);
         const uint32_t b = __ballot_sync(0xffffffffu, bit);
         if (lane == 0) bits[p] = b;
     }
 }
 
-// The warp's share (`mine` of 4) of the quarter's triplets [t0, t1).
+// The warp's share (`mine` of 4) of the triplets [t0, t1) that its quarter holds.
 template <bool kWeighted>
 __device__ __forceinline__ void eval_quarter(const LaneTriplets& tt, const PatchWeights& pw, int quarter, int mine,
-                                             int t0, int t1, uint32_t tm, uint32_t nr, const uint32_t* ext,
-                                             uint32_t* bits, int lane) {
+                                             int t0, int t1, uint32_t tm, uint32_t nr, uint32_t* bits, int lane) {
     const int16_t* start = tt.start[quarter];
-    int lo = start[0];
     if (!kWeighted && t1 - t0 == kBits) {
         eval_class<0>(tt, start[0], start[1], mine, tm, nr, bits, lane);
         eval_class<1>(tt, start[1], start[2], mine, tm, nr, bits, lane);
@@ -441,10 +432,10 @@ __device__ __forceinline__ void eval_quarter(const LaneTriplets& tt, const Patch
         eval_class<4>(tt, start[4], start[5], mine, tm, nr, bits, lane);
         eval_class<5>(tt, start[5], start[6], mine, tm, nr, bits, lane);
         eval_class<6>(tt, start[6], start[7], mine, tm, nr, bits, lane);
-        eval_class<7>(tt, start[7], start[8], mine, tm, nr, bits, lane);
-        lo = start[8];
+        eval_class<7>(tt, start[7], start[kStaged], mine, tm, nr, bits, lane);
+    } else {
+        eval_entries<kWeighted, false>(tt, pw, start[0], start[kStaged], mine, t0, t1, tm, nr, nullptr, bits, lane);
     }
-    eval_entries<kWeighted>(tt, pw, lo, start[9], start[8], mine, t0, t1, tm, nr, ext, bits, lane);
 }
 
 // Copies kRows rows (from row r of the quarter on) of the lane's staged window into the
@@ -490,7 +481,6 @@ __global__ void __launch_bounds__(kThreads, 1) extract_lanes_kernel(
     __shared__ LanesSmem S;
     uint8_t* ring = smem_raw + (-smem_u32(smem_raw) & 127u);
     uint32_t* s_stage = reinterpret_cast<uint32_t*>(ring + kRingBytes);  // [kBatch][kStageWords]
-    uint32_t* s_ext = s_stage + kBatch * kStageWords;                        // [2][kBatch][kExtWords]
     const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     volatile int* abort = &S.abort;
     if (threadIdx.x == 0) {
@@ -541,7 +531,6 @@ __global__ void __launch_bounds__(kThreads, 1) extract_lanes_kernel(
         const int cx = 4 * wi + (lane & 3), yl = lane >> 2;
         const uint32_t ring_addr = smem_u32(ring);
         const uint32_t stage_addr = smem_u32(s_stage) + 4u * static_cast<uint32_t>(cx * kWin + yl);
-        const uint32_t ext_addr = smem_u32(s_ext) + 4u * static_cast<uint32_t>((yl - (8 - kExtRows)) * kWordCols + cx);
         int seq0 = 0;        // sequence number of the item's first keypoint
         bool ok = true;
         bool primed = false; // tab holds the group's next keypoint
@@ -582,8 +571,6 @@ __global__ void __launch_bounds__(kThreads, 1) extract_lanes_kernel(
                     tab[q] = __ldg(next_tab + q * (kGroupWarps * kBlockWords));
                     const uint32_t v = __byte_perm(__byte_perm(b0, b1, 0x0040), __byte_perm(b2, b3, 0x0040), 0x5410);
                     sts_u32(to + 32u * q, v);
-                    if (q == kWarpBlocks - 1 && yl >= 8 - kExtRows)  // rows 42..47
-                        sts_u32(ext_addr + 4u * kExtWords * static_cast<uint32_t>((i & 1) * kBatch + j), v);
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&S.empty[slot]);  // the tile is free for this warp
@@ -708,6 +695,9 @@ __global__ void __launch_bounds__(kThreads, 1) extract_lanes_kernel(
     bool dead = false;  // after a failed wait: barriers without work, so that every warp reaches them
     for (int i = 0; i < S.work.items; ++i) {
         const Item it = S.work.item(i);
+        uint32_t* bits = S.bits[i & 1];
+        const int mine = (warp >> 2) & 3;
+        const int t0 = __shfl_sync(0xffffffffu, 8 * it.ca, 0), t1 = __shfl_sync(0xffffffffu, 8 * it.cb, 0);
         if (!dead) dead = !__all_sync(0xffffffffu, mbar_wait_sleep<100>(&S.staged, i & 1, abort));
         if (!dead) {
             // copy the staged windows (lane = keypoint) into this quarter, 12 rows per warp
@@ -718,20 +708,19 @@ __global__ void __launch_bounds__(kThreads, 1) extract_lanes_kernel(
             else
                 copy_rows<6>(s_stage + lane * kStageWords, Q, r0, tm);
             tmem_st_wait();
+            // ---- Eq. 1: this warp's share of the triplets that are read from the staged windows ----
+            const int16_t* start = tt.start[quarter];
+            eval_entries<kWeighted, true>(tt, pw, start[kStaged], start[kTripClasses], mine, t0, t1, tm, nr,
+                                          s_stage + lane * kStageWords, bits, lane);
             __syncwarp();
             if (lane == 0) mbar_arrive(&S.copied);
         }
         tc_fence_before();
         bar_sync_id(1 + quarter, 128);
         tc_fence_after();
-        uint32_t* bits = S.bits[i & 1];
         const int n = it.cb - it.ca;
-        if (!dead) {
-            // ---- Eq. 1: this warp's share of the quarter's triplets in the chunks [ca, cb) ----
-            const uint32_t* ext = s_ext + (i & 1) * (kBatch * kExtWords) + lane * kExtWords;
-            const int t0 = __shfl_sync(0xffffffffu, 8 * it.ca, 0), t1 = __shfl_sync(0xffffffffu, 8 * it.cb, 0);
-            eval_quarter<kWeighted>(tt, pw, quarter, (warp >> 2) & 3, t0, t1, tm, nr, ext, bits, lane);
-        }
+        // ---- and of those that the quarter holds, in the chunks [ca, cb) ----
+        if (!dead) eval_quarter<kWeighted>(tt, pw, quarter, mine, t0, t1, tm, nr, bits, lane);
         tc_fence_before();
         // all bits of the item are there, and (the buffers alternate) everybody is done with
         // the other buffer
@@ -877,31 +866,42 @@ static bool patch_in(const Quarter& Q, int x0, int y0, int size) {
 // costs least, with as many triplets in each as their fits allow.
 void plan_triplets(const latch_triplet* trip, int size, LaneTripletPlan* plan) {
     // clocks of triplet t in quarter q (as measured): more with every patch that does not
-    // start at a word, and most with rows from shared memory; < 0: does not fit
-    constexpr int kCost = 72, kShiftCost = 9, kExtCost = 230;
+    // start at a word (plain patches), most from the staged windows
+    const int kCost = size == 8 ? 800 : 72, kShiftCost = size == 8 ? 0 : 9, kStagedCost = size == 8 ? 950 : 250;
+    constexpr int kBuildCost = 10000;  // of a batch's windows, after the triplets read from the staged ones
     int cost[kBits][kQuarters];
+    bool held[kBits][kQuarters], fixed[kBits];
     int8_t in[kBits];
-    int load[kQuarters] = {};
+    int load[kQuarters] = {}, staged[kQuarters] = {};  // clocks in all, and from the staged windows
+    int nowhere = 0;
     for (int t = 0; t < kBits; ++t) {
         const uint8_t* c = &trip[t].ax;
+        in[t] = 0;
+        fixed[t] = true;
         for (int q = 0; q < kQuarters; ++q) {
             const Quarter Q = quarter_of(q);
             int shifts = 0;
-            bool all = true;
+            held[t][q] = true;
             for (int p = 0; p < 3; ++p) {
                 const int x0 = c[2 * p] - kPatchR, y0 = c[2 * p + 1] - kPatchR;
-                all = all && patch_in(Q, x0, y0, size);
+                held[t][q] = held[t][q] && patch_in(Q, x0, y0, size);
                 shifts += ((x0 - Q.b0) & 3) != 0;
             }
-            cost[t][q] = all ? kCost + shifts * kShiftCost : q == 0 ? kCost + 3 * kShiftCost + kExtCost : -1;
+            cost[t][q] = held[t][q] ? kCost + shifts * kShiftCost : kStagedCost;
+            if (cost[t][q] < cost[t][in[t]]) in[t] = static_cast<int8_t>(q);
+            fixed[t] = fixed[t] && !held[t][q];
         }
-        in[t] = 0;
-        for (int q = 1; q < kQuarters; ++q)
-            if (cost[t][q] >= 0 && cost[t][q] < cost[t][in[t]]) in[t] = static_cast<int8_t>(q);
+        // plain ones that no quarter holds go round: the builders wait for them (weighted ones
+        // take long enough next to the building)
+        fixed[t] = fixed[t] && size != 8;
+        if (fixed[t]) in[t] = static_cast<int8_t>(nowhere++ % kQuarters);
         load[in[t]] += cost[t][in[t]];
+        if (!held[t][in[t]]) staged[in[t]] += kStagedCost;
     }
-    // move triplets between quarters, each time the move that costs least among those out
-    // of the fullest quarter that has one (one that lowers the load of the two)
+    // move the others between quarters, each time the move that costs least among those out
+    // of the fullest quarter that has one: it lowers the load of the two, and what a quarter
+    // reads from the staged windows and the next batch's building, which waits for it, stay
+    // below that load
     for (int moves = 0; moves < 4 * kBits; ++moves) {
         int best = -1, to = 0, least = 0;
         int below = INT32_MAX;
@@ -911,9 +911,11 @@ void plan_triplets(const latch_triplet* trip, int size, LaneTripletPlan* plan) {
                 if (load[q] < below && (full < 0 || load[q] > load[full])) full = q;
             if (full < 0) break;
             below = load[full];
-            for (int t = 0; t < kBits; ++t)
+            for (int k = 0; k < kBits; ++k)
                 for (int q = 0; q < kQuarters; ++q) {
-                    if (in[t] != full || cost[t][q] < 0 || load[q] + cost[t][q] >= load[full]) continue;
+                    const int t = k * 317 & (kBits - 1);  // spread over the indices, so over the chunks
+                    if (in[t] != full || fixed[t] || load[q] + cost[t][q] >= load[full]) continue;
+                    if (!held[t][q] && staged[q] + kStagedCost + kBuildCost >= load[full]) continue;
                     const int d = cost[t][q] - cost[t][full];
                     if (best < 0 || d < least) {
                         best = t;
@@ -923,14 +925,16 @@ void plan_triplets(const latch_triplet* trip, int size, LaneTripletPlan* plan) {
                 }
         }
         if (best < 0) break;
-        load[in[best]] -= cost[best][in[best]];
+        const int from = in[best];
+        load[from] -= cost[best][from];
         load[to] += cost[best][to];
+        if (!held[best][from]) staged[from] -= kStagedCost;
+        if (!held[best][to]) staged[to] += kStagedCost;
         in[best] = static_cast<int8_t>(to);
     }
     int at = 0;
     for (int q = 0; q < kQuarters; ++q) {
         const Quarter Q = quarter_of(q);
-        uint32_t word[3];
         for (int cls = 0; cls < kTripClasses; ++cls) {
             plan->start[q][cls] = static_cast<int16_t>(at);
             for (int t = 0; t < kBits; ++t) {
@@ -938,14 +942,18 @@ void plan_triplets(const latch_triplet* trip, int size, LaneTripletPlan* plan) {
                 const uint8_t* c = &trip[t].ax;
                 int own = 0;
                 for (int p = 0; p < 3; ++p) {
-                    const int x0 = c[2 * p] - kPatchR - Q.b0, y0 = c[2 * p + 1] - kPatchR - Q.r0;
-                    word[p] = static_cast<uint32_t>(8 * (x0 & 3)) | static_cast<uint32_t>((x0 >> 2) * Q.nr + y0) << 16;
-                    own |= (x0 & 3) ? 1 << p : 0;
-                    if (!patch_in(Q, c[2 * p] - kPatchR, c[2 * p + 1] - kPatchR, size)) own |= 8;
+                    const int x0 = c[2 * p] - kPatchR, y0 = c[2 * p + 1] - kPatchR;
+                    own |= ((x0 - Q.b0) & 3) ? 1 << p : 0;
+                    if (!patch_in(Q, x0, y0, size)) own |= kStaged;
                 }
-                if ((own & 8 ? 8 : own) != cls) continue;
-                word[0] |= static_cast<uint32_t>(t) << 5;
-                for (int p = 0; p < 3; ++p) plan->e[p][at] = word[p];
+                if ((own & kStaged ? kStaged : own) != cls) continue;
+                const Quarter from = cls == kStaged ? Quarter{0, kWordCols, 0, kWin} : Q;
+                for (int p = 0; p < 3; ++p) {
+                    const int x = c[2 * p] - kPatchR - from.b0, y = c[2 * p + 1] - kPatchR - from.r0;
+                    plan->e[p][at] = static_cast<uint32_t>(8 * (x & 3)) |
+                                     static_cast<uint32_t>((x >> 2) * from.nr + y) << 16 |
+                                     (p == 0 ? static_cast<uint32_t>(t) << 5 : 0u);
+                }
                 ++at;
             }
         }
