@@ -861,103 +861,156 @@ static bool patch_in(const Quarter& Q, int x0, int y0, int size) {
            ((x & 3) == 0 || ((x >> 2) + 2) * Q.nr + y <= kTmLast);
 }
 
+// The quarters (bit q) that hold the patch at (x0, y0).
+struct PatchMasks {
+    uint8_t at[kWin][kWin];
+    explicit PatchMasks(int size) {
+        for (int y = 0; y < kWin; ++y)
+            for (int x = 0; x < kWin; ++x) {
+                at[y][x] = 0;
+                for (int q = 0; q < kQuarters; ++q)
+                    at[y][x] |= static_cast<uint8_t>(patch_in(quarter_of(q), x, y, size) << q);
+            }
+    }
+};
+
+// Sets of the triplets that could move: bit k is triplet order(k).
+struct TripletSet {
+    uint64_t w[kBits / 64];
+    int n;
+    void add(int k) { w[k >> 6] |= uint64_t(1) << (k & 63), ++n; }
+    void remove(int k) { w[k >> 6] &= ~(uint64_t(1) << (k & 63)), --n; }
+    int first() const {
+        int i = 0;
+        while (!w[i]) ++i;
+        return 64 * i + __builtin_ctzll(w[i]);
+    }
+};
+
 // The triplet table as the evaluators read it (LaneTriplets) for patches of `size` x
 // `size` pixels (7, or 8 when weighted): every triplet goes to the quarter in which it
-// costs least, with as many triplets in each as their fits allow.
+// costs least, and then moves between quarters level their loads.  latch_extract plans
+// whenever it is given another table than before, so a move takes the first of the sets of
+// triplets that it costs the same, not a search of the table (that took 0.2-0.5 ms of host
+// time a table, this 20-60 us: calls of 2,000 keypoints that alternate between two tables
+// 253 -> 50 us each, with one table 37).
 void plan_triplets(const latch_triplet* trip, int size, LaneTripletPlan* plan) {
-    // clocks of triplet t in quarter q (as measured): more with every patch that does not
-    // start at a word (plain patches), most from the staged windows
-    const int kCost = size == 8 ? 800 : 72, kShiftCost = size == 8 ? 0 : 9, kStagedCost = size == 8 ? 950 : 250;
+    static const PatchMasks masks7(2 * kPatchR + 1), masks8(2 * kPatchR + 2);
+    const PatchMasks& masks = size == 8 ? masks8 : masks7;
+    // clocks of a triplet (as measured) by its level in a quarter: more with every patch that
+    // does not start at a word (level = their number; the same for weighted patches), most
+    // from the staged windows
+    constexpr int kLevels = 5, kStagedLevel = 4;
+    const int plain[kLevels] = {72, 81, 90, 99, 250}, weighted[kLevels] = {800, 800, 800, 800, 950};
+    const int* cost = size == 8 ? weighted : plain;
     constexpr int kBuildCost = 10000;  // of a batch's windows, after the triplets read from the staged ones
-    int cost[kBits][kQuarters];
-    bool held[kBits][kQuarters], fixed[kBits];
-    int8_t in[kBits];
+    auto order = [](int k) { return k * 317 & (kBits - 1); };  // spread over the indices, so over the chunks
+    uint8_t level[kBits][kQuarters], in[kBits];
     int load[kQuarters] = {}, staged[kQuarters] = {};  // clocks in all, and from the staged windows
     int nowhere = 0;
-    for (int t = 0; t < kBits; ++t) {
+    TripletSet sets[kQuarters][kLevels][kQuarters][kLevels] = {};  // [quarter][level there][other quarter][level there]
+    auto each_set = [&](int k, auto&& f) {
+        const int t = order(k), q = in[t];
+        for (int o = 0; o < kQuarters; ++o)
+            if (o != q) f(sets[q][level[t][q]][o][level[t][o]], k);
+    };
+    for (int k = 0; k < kBits; ++k) {
+        const int t = order(k);
         const uint8_t* c = &trip[t].ax;
-        in[t] = 0;
-        fixed[t] = true;
+        uint32_t held = 15;
+        for (int p = 0; p < 3; ++p) held &= masks.at[c[2 * p + 1] - kPatchR][c[2 * p] - kPatchR];
+        int best = 0;
         for (int q = 0; q < kQuarters; ++q) {
-            const Quarter Q = quarter_of(q);
-            int shifts = 0;
-            held[t][q] = true;
-            for (int p = 0; p < 3; ++p) {
-                const int x0 = c[2 * p] - kPatchR, y0 = c[2 * p + 1] - kPatchR;
-                held[t][q] = held[t][q] && patch_in(Q, x0, y0, size);
-                shifts += ((x0 - Q.b0) & 3) != 0;
-            }
-            cost[t][q] = held[t][q] ? kCost + shifts * kShiftCost : kStagedCost;
-            if (cost[t][q] < cost[t][in[t]]) in[t] = static_cast<int8_t>(q);
-            fixed[t] = fixed[t] && !held[t][q];
+            const int b0 = quarter_of(q).b0 + kPatchR;
+            const int shifts = (((c[0] - b0) & 3) != 0) + (((c[2] - b0) & 3) != 0) + (((c[4] - b0) & 3) != 0);
+            level[t][q] = static_cast<uint8_t>(held >> q & 1 ? shifts : kStagedLevel);
+            if (cost[level[t][q]] < cost[level[t][best]]) best = q;
         }
-        // plain ones that no quarter holds go round: the builders wait for them (weighted ones
-        // take long enough next to the building)
-        fixed[t] = fixed[t] && size != 8;
-        if (fixed[t]) in[t] = static_cast<int8_t>(nowhere++ % kQuarters);
-        load[in[t]] += cost[t][in[t]];
-        if (!held[t][in[t]]) staged[in[t]] += kStagedCost;
+        // plain ones that no quarter holds go round and stay: the builders wait for them
+        // (weighted ones take long enough next to the building)
+        const bool fixed = !held && size != 8;
+        if (fixed) best = nowhere++ % kQuarters;
+        in[t] = static_cast<uint8_t>(best);
+        load[best] += cost[level[t][best]];
+        if (level[t][best] == kStagedLevel) staged[best] += cost[kStagedLevel];
+        if (!fixed) each_set(k, [](TripletSet& s, int i) { s.add(i); });
     }
-    // move the others between quarters, each time the move that costs least among those out
-    // of the fullest quarter that has one: it lowers the load of the two, and what a quarter
-    // reads from the staged windows and the next batch's building, which waits for it, stay
-    // below that load
+    // the changes of level by what they cost
+    struct Change {
+        int from, to, d;
+    } changes[kLevels * kLevels];
+    for (int i = 0; i < kLevels * kLevels; ++i) {
+        const Change c{i / kLevels, i % kLevels, cost[i % kLevels] - cost[i / kLevels]};
+        int j = i;
+        for (; j > 0 && changes[j - 1].d > c.d; --j) changes[j] = changes[j - 1];
+        changes[j] = c;
+    }
+    // each time the move that costs least among those out of the fullest quarter that has one:
+    // it lowers the load of the two, and what a quarter reads from the staged windows and the
+    // next batch's building, which waits for it, stay below that load
     for (int moves = 0; moves < 4 * kBits; ++moves) {
-        int best = -1, to = 0, least = 0;
+        int move = -1, to = 0;
         int below = INT32_MAX;
-        while (best < 0) {
+        while (move < 0) {
             int full = -1;
             for (int q = 0; q < kQuarters; ++q)
                 if (load[q] < below && (full < 0 || load[q] > load[full])) full = q;
             if (full < 0) break;
             below = load[full];
-            for (int k = 0; k < kBits; ++k)
+            int least = 0;
+            for (const Change& c : changes) {
+                if (move >= 0 && c.d > least) break;
                 for (int q = 0; q < kQuarters; ++q) {
-                    const int t = k * 317 & (kBits - 1);  // spread over the indices, so over the chunks
-                    if (in[t] != full || fixed[t] || load[q] + cost[t][q] >= load[full]) continue;
-                    if (!held[t][q] && staged[q] + kStagedCost + kBuildCost >= load[full]) continue;
-                    const int d = cost[t][q] - cost[t][full];
-                    if (best < 0 || d < least) {
-                        best = t;
-                        to = q;
-                        least = d;
-                    }
+                    const TripletSet& s = sets[full][c.from][q][c.to];
+                    if (s.n == 0 || load[q] + cost[c.to] >= load[full]) continue;
+                    if (c.to == kStagedLevel && staged[q] + cost[kStagedLevel] + kBuildCost >= load[full]) continue;
+                    const int k = s.first();
+                    if (move >= 0 && k >= move) continue;
+                    move = k;
+                    to = q;
+                    least = c.d;
                 }
-        }
-        if (best < 0) break;
-        const int from = in[best];
-        load[from] -= cost[best][from];
-        load[to] += cost[best][to];
-        if (!held[best][from]) staged[from] -= kStagedCost;
-        if (!held[best][to]) staged[to] += kStagedCost;
-        in[best] = static_cast<int8_t>(to);
-    }
-    int at = 0;
-    for (int q = 0; q < kQuarters; ++q) {
-        const Quarter Q = quarter_of(q);
-        for (int cls = 0; cls < kTripClasses; ++cls) {
-            plan->start[q][cls] = static_cast<int16_t>(at);
-            for (int t = 0; t < kBits; ++t) {
-                if (in[t] != q) continue;
-                const uint8_t* c = &trip[t].ax;
-                int own = 0;
-                for (int p = 0; p < 3; ++p) {
-                    const int x0 = c[2 * p] - kPatchR, y0 = c[2 * p + 1] - kPatchR;
-                    own |= ((x0 - Q.b0) & 3) ? 1 << p : 0;
-                    if (!patch_in(Q, x0, y0, size)) own |= kStaged;
-                }
-                if ((own & kStaged ? kStaged : own) != cls) continue;
-                const Quarter from = cls == kStaged ? Quarter{0, kWordCols, 0, kWin} : Q;
-                for (int p = 0; p < 3; ++p) {
-                    const int x = c[2 * p] - kPatchR - from.b0, y = c[2 * p + 1] - kPatchR - from.r0;
-                    plan->e[p][at] = static_cast<uint32_t>(8 * (x & 3)) |
-                                     static_cast<uint32_t>((x >> 2) * from.nr + y) << 16 |
-                                     (p == 0 ? static_cast<uint32_t>(t) << 5 : 0u);
-                }
-                ++at;
             }
         }
+        if (move < 0) break;
+        const int t = order(move), from = in[t];
+        each_set(move, [](TripletSet& s, int i) { s.remove(i); });
+        load[from] -= cost[level[t][from]];
+        if (level[t][from] == kStagedLevel) staged[from] -= cost[kStagedLevel];
+        in[t] = static_cast<uint8_t>(to);
+        load[to] += cost[level[t][to]];
+        if (level[t][to] == kStagedLevel) staged[to] += cost[kStagedLevel];
+        each_set(move, [](TripletSet& s, int i) { s.add(i); });
+    }
+    // the list, by quarter, class and index
+    uint8_t cls[kBits];
+    int count[kQuarters][kTripClasses] = {}, at = 0;
+    for (int t = 0; t < kBits; ++t) {
+        const uint8_t* c = &trip[t].ax;
+        const int b0 = quarter_of(in[t]).b0 + kPatchR;
+        cls[t] = kStaged;
+        if (level[t][in[t]] != kStagedLevel)
+            cls[t] = static_cast<uint8_t>((((c[0] - b0) & 3) != 0) | (((c[2] - b0) & 3) != 0) << 1 |
+                                          (((c[4] - b0) & 3) != 0) << 2);
+        ++count[in[t]][cls[t]];
+    }
+    for (int q = 0; q < kQuarters; ++q) {
+        for (int i = 0; i < kTripClasses; ++i) {
+            plan->start[q][i] = static_cast<int16_t>(at);
+            at += count[q][i];
+            count[q][i] = plan->start[q][i];  // from here on: the next entry
+        }
         plan->start[q][kTripClasses] = static_cast<int16_t>(at);
+    }
+    for (int t = 0; t < kBits; ++t) {
+        const uint8_t* c = &trip[t].ax;
+        const Quarter from = cls[t] == kStaged ? Quarter{0, kWordCols, 0, kWin} : quarter_of(in[t]);
+        const int e = count[in[t]][cls[t]]++;
+        for (int p = 0; p < 3; ++p) {
+            const int x = c[2 * p] - kPatchR - from.b0, y = c[2 * p + 1] - kPatchR - from.r0;
+            plan->e[p][e] = static_cast<uint32_t>(8 * (x & 3)) | static_cast<uint32_t>((x >> 2) * from.nr + y) << 16 |
+                            (p == 0 ? static_cast<uint32_t>(t) << 5 : 0u);
+        }
     }
 }
 

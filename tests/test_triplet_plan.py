@@ -3,6 +3,7 @@ triplet once, its patches from the quarter's part of the window or from the stag
 the work spread over the four quarters (each is one SM partition) also for tables whose patches
 lie far apart."""
 import ctypes
+import time
 
 import numpy as np
 import pytest
@@ -75,3 +76,16 @@ def test_plan(plan_triplets, kind, size):
                         assert (x & 3) == 0 or ((x >> 2) + 2) * nr + y <= LAST_COLUMN
     # a quarter is one SM partition: none may take more than half of the triplets
     assert (start[:, CLASSES] - start[:, 0]).max() <= BITS // 2
+
+
+@pytest.mark.parametrize("size", [7, 8])
+@pytest.mark.parametrize("kind", ["seeded", "uniform", "last_rows"])
+def test_plan_is_quick(plan_triplets, kind, size):
+    """An extraction that is given another table than the last one plans it first: that has
+    to stay small next to a launch (best of many runs, below 0.1 ms on any host)."""
+    t, plan, best = table(kind, size), Plan(), 1.0
+    for _ in range(50):
+        t0 = time.perf_counter()
+        plan_triplets(t.ctypes.data, size, ctypes.byref(plan))
+        best = min(best, time.perf_counter() - t0)
+    assert best < 1e-4
