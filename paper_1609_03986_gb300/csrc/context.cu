@@ -115,12 +115,19 @@ static latch_status upload_scales(latch_context* ctx, const double* scales, int 
 // needs about 18 us for a tile's rows whatever the query count and merges the tiles in a
 // second launch, the tensor path 12 us with its expansion (300 x 300: 18.5 against 11.8
 // us, 2,000 x 2,000: 28.4 / 14.5, 100 x 10,000: 30.8 / 24.1; up to 256 rows 10,000 x 100:
-// 10.3 / 12.0, 50,000 x 20: 8.5 / 24.0).  Beyond 65,536 train rows the pair count decides
-// alone: the path's scratch is 256 bytes per row.
+// 10.3 / 12.0, 50,000 x 20: 8.5 / 24.0).  A few queries against 17,000 to 30,000 rows
+// stay: on the CUDA cores each tile has an SM, while on the tensor cores every block pair
+// walks a unit of the same query tile and the last one combines 60 to 76 records a row (1 x
+// 20,000: 30.9 / 36.7, 6 x 30,000 35.0 / 37.8, 8 x 24,000 35.2 / 37.4; about equal at 8 x 28,000
+// and 12 x 24,000; 4 x 34,000 40.1 / 38.1, 16 x 26,000 39.1 / 37.4).  Beyond 65,536 rows the pair
+// count decides alone, although the tensor cores are faster there too (30 x 140,000 309 / 51):
+// the path's scratch is 256 bytes per row, and the context keeps it -- a gigabyte for a single
+// query against 2^22 rows, which such a call never took.
 static int choose_match_path(const latch_context* ctx, int64_t nq, int64_t nt) {
     if (nq * nt >= ctx->tensor_min_pairs) return LATCH_PATH_TENSOR;
     const bool small = ctx->tensor_min_pairs == kDefaultTensorMinPairs && nt > 256 && nt <= 65536;
-    return small ? LATCH_PATH_TENSOR : LATCH_PATH_POPC;
+    const bool few = nq <= 12 && nt > 17000 && nt <= 30000 && nt <= 36000 - 1000 * nq;
+    return small && !few ? LATCH_PATH_TENSOR : LATCH_PATH_POPC;
 }
 
 // Triplet coordinates must keep every patch inside the 48x48 window: [3, 44] for the
