@@ -387,9 +387,7 @@ const char *latch_session_last_error(const latch_session *s);
 /* ---- Autotuning (tile shapes and path choice, by measurement on this device) ---- */
 typedef struct {
     int32_t item_kps;           /* extraction: fewest keypoints per batch (one block builds their windows), 1..32 */
-    int64_t tensor_min_pairs;   /* matching: LATCH_PATH_AUTO uses the tensor cores from nq*nt >= this (at its
-                                 * default, 2^22, also for smaller problems of 257 to 65,536 train rows, but for
-                                 * up to 12 queries against 17,000 to 30,000) */
+    int64_t tensor_min_pairs;   /* matching: LATCH_PATH_AUTO uses the tensor cores from nq*nt >= this */
 } latch_tuning;
 
 typedef struct {
@@ -397,6 +395,12 @@ typedef struct {
     int32_t n_keypoints;        /* keypoints per image (0: skip the extraction tuning) */
     int32_t n_query, n_train;   /* representative matching shape (0: skip the matching tuning) */
 } latch_tune_shape;
+
+/* By default tensor_min_pairs is 2^22 and AUTO uses the tensor cores for smaller problems of
+ * 257 to 65,536 train rows too, but for up to 12 queries against 17,000 to 30,000 rows.
+ * latch_autotune keeps that rule for smaller problems unless it measures the contrary;
+ * latch_set_tuning with 2^22 restores it, and with any other value than the context's own
+ * sets a plain threshold. */
 
 /* Measure the candidate extraction batch sizes and the matching paths on
  * synthetic device data of this shape and keep the fastest in the context; results

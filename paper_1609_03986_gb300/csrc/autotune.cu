@@ -1,11 +1,11 @@
-// Autotuner: picks, by measurement on this device, (1) the fewest keypoints an
-// extraction block takes (which sets the grid on small inputs) and (2) the pair count
-// from which LATCH_PATH_AUTO matches on
-// the tensor cores instead of the CUDA cores.  It runs on synthetic device data
+// Autotuner: picks, by measurement on this device, (1) the fewest keypoints of an
+// extraction batch (whose windows one block builds) and (2) the pair count from which
+// LATCH_PATH_AUTO matches on the tensor cores instead of the CUDA cores, and whether smaller
+// problems go to the tensor cores as they do by default.  It runs on synthetic device data
 // shaped like the caller's workload (image size, keypoints, query and train counts),
 // times every candidate with CUDA events (median of 3 after a warm-up), and stores
 // the winners in the context.  latch_get_tuning / latch_set_tuning read and restore
-// them, so a caller can cache them per device.
+// the numbers, so a caller can cache them per device.
 #include <algorithm>
 #include <vector>
 
@@ -74,6 +74,22 @@ float median_ms(F&& run, cudaStream_t s) {
 }
 
 }  // namespace
+
+// The threshold is the pair count of the first rung on which the tensor path wins.  The
+// default rule for smaller problems stays unless a rung of its range was measured the other
+// way.  2^22, the value that latch_set_tuning takes for threshold and rule together, is left
+// to mean that.
+void tuned_matching(int64_t nq, const MatchRung* rungs, int n, int64_t* min_pairs, bool* small) {
+    *small = true;
+    int first = n;
+    for (int i = n - 1; i >= 0; --i) {
+        if (rungs[i].tensor_wins) first = i;
+        else if (small_problem_to_tensor(nq, rungs[i].nt)) *small = false;
+    }
+    *min_pairs = first < n ? nq * rungs[first].nt : nq * rungs[n - 1].nt * 4;
+    if (!*small && *min_pairs == kDefaultTensorMinPairs) *min_pairs += first < n ? -1 : 1;
+}
+
 }  // namespace latch
 
 using namespace latch;
@@ -92,6 +108,10 @@ latch_status latch_set_tuning(latch_context* ctx, const latch_tuning* t) {
     if (t->item_kps < 1 || t->item_kps > 32 || t->tensor_min_pairs < 0)
         return fail(ctx, LATCH_EINVAL, "item_kps must be in [1, 32], tensor_min_pairs >= 0");
     ctx->item_kps = t->item_kps;
+    // the default value brings the rule for smaller problems with it; a context that is given
+    // its own value again stays as it is
+    if (t->tensor_min_pairs != ctx->tensor_min_pairs)
+        ctx->small_to_tensor = t->tensor_min_pairs == kDefaultTensorMinPairs;
     ctx->tensor_min_pairs = t->tensor_min_pairs;
     return LATCH_OK;
 }
@@ -107,7 +127,7 @@ latch_status latch_autotune(latch_context* ctx, const latch_tune_shape* shape, l
     cudaStream_t s = nullptr;
     LATCH_CUDA_TRY(ctx, cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
     latch_status st = LATCH_OK;
-    // ---- extraction: fewest keypoints per block ----
+    // ---- extraction: fewest keypoints per batch ----
     if (sh.n_keypoints > 0) {
         const int64_t pitch = (static_cast<int64_t>(sh.width) + 15) / 16 * 16;
         uint8_t *img = nullptr, *out_desc = nullptr;
@@ -160,9 +180,9 @@ latch_status latch_autotune(latch_context* ctx, const latch_tune_shape* shape, l
             note_launches(2);
             e = cudaGetLastError();
         }
-        // ladder of train-set sizes (the query set fixed): the smallest size at
-        // which the tensor path wins sets the pair threshold
-        int64_t threshold = -1;
+        // ladder of train-set sizes (the query set fixed), up to the first on which the tensor
+        // path wins
+        std::vector<MatchRung> rungs;
         for (int64_t ntr = std::min<int64_t>(nt, 64); e == cudaSuccess && st == LATCH_OK; ntr *= 4) {
             if (ntr > nt) ntr = nt;
             float ms[2] = {0.f, 0.f};
@@ -174,13 +194,13 @@ latch_status latch_autotune(latch_context* ctx, const latch_tune_shape* shape, l
                                            paths[k], s);
                     },
                     s);
-            if (st == LATCH_OK && ms[1] <= ms[0]) {
-                threshold = nq * ntr;
-                break;
-            }
-            if (ntr == nt) break;
+            if (st != LATCH_OK) break;
+            rungs.push_back(MatchRung{ntr, ms[1] <= ms[0]});
+            if (rungs.back().tensor_wins || ntr == nt) break;
         }
-        if (st == LATCH_OK) ctx->tensor_min_pairs = threshold >= 0 ? threshold : nq * nt * 4;
+        if (st == LATCH_OK && !rungs.empty())
+            tuned_matching(nq, rungs.data(), static_cast<int>(rungs.size()), &ctx->tensor_min_pairs,
+                           &ctx->small_to_tensor);
         if (q) cudaFree(q);
         if (t) cudaFree(t);
         if (m) cudaFree(m);

@@ -110,8 +110,9 @@ static latch_status upload_scales(latch_context* ctx, const double* scales, int 
 }
 
 // Matching path for AUTO: the tensor cores from tensor_min_pairs pairs on
-// (latch_autotune, latch_set_tuning).  At its default value they also take smaller
-// problems of more than one CUDA-core train tile (256 rows): a block of the CUDA cores
+// (latch_autotune, latch_set_tuning).  By default, and after an autotuning that does not
+// measure the contrary, they also take smaller problems of more than one CUDA-core train
+// tile (256 rows): a block of the CUDA cores
 // needs about 18 us for a tile's rows whatever the query count and merges the tiles in a
 // second launch, the tensor path 12 us with its expansion (300 x 300: 18.5 against 11.8
 // us, 2,000 x 2,000: 28.4 / 14.5, 100 x 10,000: 30.8 / 24.1; up to 256 rows 10,000 x 100:
@@ -123,11 +124,15 @@ static latch_status upload_scales(latch_context* ctx, const double* scales, int 
 // count decides alone, although the tensor cores are faster there too (30 x 140,000 309 / 51):
 // the path's scratch is 256 bytes per row, and the context keeps it -- a gigabyte for a single
 // query against 2^22 rows, which such a call never took.
-static int choose_match_path(const latch_context* ctx, int64_t nq, int64_t nt) {
-    if (nq * nt >= ctx->tensor_min_pairs) return LATCH_PATH_TENSOR;
-    const bool small = ctx->tensor_min_pairs == kDefaultTensorMinPairs && nt > 256 && nt <= 65536;
+bool small_problem_to_tensor(int64_t nq, int64_t nt) {
     const bool few = nq <= 12 && nt > 17000 && nt <= 30000 && nt <= 36000 - 1000 * nq;
-    return small && !few ? LATCH_PATH_TENSOR : LATCH_PATH_POPC;
+    return nt > 256 && nt <= 65536 && !few;
+}
+
+static int choose_match_path(const latch_context* ctx, int64_t nq, int64_t nt) {
+    const bool tensor =
+        nq * nt >= ctx->tensor_min_pairs || (ctx->small_to_tensor && small_problem_to_tensor(nq, nt));
+    return tensor ? LATCH_PATH_TENSOR : LATCH_PATH_POPC;
 }
 
 // Triplet coordinates must keep every patch inside the 48x48 window: [3, 44] for the

@@ -48,6 +48,17 @@ __device__ __forceinline__ uint4 expand_word_e2m1(uint32_t w) {
 
 constexpr int64_t kDefaultTensorMinPairs = int64_t(1) << 22;
 
+// What latch_autotune keeps of a ladder of train-set sizes (`rungs`, the last one the whole
+// set) against nq queries, on which each path was timed: the pair threshold of LATCH_PATH_AUTO,
+// and whether smaller problems go to the tensor cores as they do by default.
+struct MatchRung {
+    int64_t nt;
+    bool tensor_wins;
+};
+void tuned_matching(int64_t nq, const MatchRung* rungs, int n, int64_t* min_pairs, bool* small);
+// Whether the default rule sends a problem below the pair threshold to the tensor cores.
+bool small_problem_to_tensor(int64_t nq, int64_t nt);
+
 // Device-side error flags (OR-ed into ctx->d_flags).
 enum : uint32_t { kFlagBadScale = 1u, kFlagTimeout = 2u };
 
@@ -98,6 +109,7 @@ struct latch_context {
     cudaEvent_t* trace_ev = nullptr;
     int32_t trace_cap = 0, trace_n = 0;
     int64_t tensor_min_pairs = latch::kDefaultTensorMinPairs;  // matching: AUTO uses the tensor path from here
+    bool small_to_tensor = true;         // and for smaller problems (choose_match_path)
     latch::Scratch scratch[4];           // grow-only: CUDA-core matching, tensor matching, batch, detection
     // latch_batch_run_host: two staging sets used alternately, upload stream
     latch::HostStaging staging[2];
