@@ -369,12 +369,16 @@ __global__ void __launch_bounds__(256) detect_expand_kernel(const DetectParams p
     }
 }
 
-// Level images of the levels with scale != 1: one thread per 16 output columns of
-// kLevelRows rows, row groups of all levels in one grid (group r of the launch is level
-// `lev`'s group r - row0[lev]).  out(x, y) = base(rha(s x), rha(s y)).  The FP64 products
-// and roundings of the columns bound the kernel when every row computed them (74 us for
-// the two levels of a 4000x3000 image); the rows of a group share them.
+// Level images of the levels with scale != 1: one thread per 16 output columns of `rows`
+// rows, row groups of all levels in one grid (group r of the launch is level `lev`'s group
+// r - row0[lev]).  out(x, y) = base(rha(s x), rha(s y)).  The FP64 products and roundings of
+// the columns bound the kernel when every row computes them (74 us for the two levels of a
+// 4000x3000 image); the rows of a group share them.  That takes threads away: groups of 8
+// rows left 1,809 threads of a 640x480 image's two levels, eight blocks (18.5 us; a row each in
+// blocks of 64 7.7), so a group has as many rows as leave kLevelThreads threads.
 constexpr int kLevelRows = 8;
+constexpr int kLevelThreads = 16384;
+constexpr int kLevelBlock = 64;
 
 struct ResampleParams {
     const uint8_t* base;
@@ -382,13 +386,14 @@ struct ResampleParams {
     uint8_t* out[kMaxDetectLevels];
     int64_t pitch[kMaxDetectLevels];
     int32_t width[kMaxDetectLevels], height[kMaxDetectLevels];
+    int32_t rows;                        // rows per group
     int32_t row0[kMaxDetectLevels + 1];  // first row group of each level; row0[n] = groups of all levels
     double scale[kMaxDetectLevels];
     int32_t n;
     int32_t chunks;  // 16-byte chunks per launch row: those of the widest level
 };
 
-__global__ void __launch_bounds__(256) pyramid_level_kernel(const ResampleParams prm) {
+__global__ void __launch_bounds__(kLevelBlock) pyramid_level_kernel(const ResampleParams prm) {
     griddep_wait();
     griddep_launch_dependents();
     const int64_t gid = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -397,7 +402,7 @@ __global__ void __launch_bounds__(256) pyramid_level_kernel(const ResampleParams
     if (row >= prm.row0[prm.n]) return;
     int l = 0;
     while (l + 1 < prm.n && prm.row0[l + 1] <= row) ++l;
-    const int y0 = static_cast<int>(row - prm.row0[l]) * kLevelRows;
+    const int y0 = static_cast<int>(row - prm.row0[l]) * prm.rows;
     const int x0 = static_cast<int>(gid % chunks_per_row) * 16;
     const int w = prm.width[l], h = prm.height[l];
     if (x0 >= w) return;
@@ -406,7 +411,7 @@ __global__ void __launch_bounds__(256) pyramid_level_kernel(const ResampleParams
 #pragma unroll
     for (int i = 0; i < 16; ++i)
         sx[i] = x0 + i < w ? static_cast<int32_t>(round(s * static_cast<double>(x0 + i))) : -1;
-    for (int y = y0; y < y0 + kLevelRows && y < h; ++y) {
+    for (int y = y0; y < y0 + prm.rows && y < h; ++y) {
         const uint8_t* src = prm.base + static_cast<int64_t>(round(s * static_cast<double>(y))) * prm.base_pitch;
         union {
             uint4 v;
@@ -493,15 +498,25 @@ cudaError_t launch_detect(const latch_image* img, const double* scales, const in
         rs.width[k] = L.width;
         rs.height[k] = L.height;
         rs.scale[k] = L.scale;
-        rs.row0[k + 1] = rs.row0[k] + (L.height + kLevelRows - 1) / kLevelRows;
         rs.chunks = std::max<int32_t>(rs.chunks, (L.width + 15) / 16);
         off += (static_cast<size_t>(L.height) * L.pitch + 255) / 256 * 256;
     }
     cudaError_t e = cudaSuccess;
     if (rs.n > 0) {
-        const int64_t threads = static_cast<int64_t>(rs.row0[rs.n]) * rs.chunks;
-        e = launch_chained(pyramid_level_kernel, dim3(static_cast<unsigned>((threads + 255) / 256)), dim3(256), 0,
-                           stream, rs);
+        int64_t threads = 0;
+        for (rs.rows = kLevelRows;; rs.rows /= 2) {
+            for (int k = 0; k < rs.n; ++k) rs.row0[k + 1] = rs.row0[k] + (rs.height[k] + rs.rows - 1) / rs.rows;
+            threads = static_cast<int64_t>(rs.row0[rs.n]) * rs.chunks;
+            if (rs.rows == 1 || threads >= kLevelThreads) break;
+        }
+        // An ordinary launch.  Launched early (launch_chained) behind a kernel that fills every SM,
+        // its blocks crowd on the first SMs that come free, whose FP64 units then hold them up
+        // (640x480, three levels without a keypoint, calls back to back: 36.9 us against 18.7,
+        // 1920x1080 53.2 / 31.3, 4000x3000 123 / 104).
+        pyramid_level_kernel<<<static_cast<unsigned>((threads + kLevelBlock - 1) / kLevelBlock), kLevelBlock, 0, stream>>>(
+            rs);
+        note_launches(1);
+        e = cudaGetLastError();
     }
     if (e != cudaSuccess) return e;
     if (ncells == 0) return cudaMemsetAsync(d_count, 0, sizeof(int32_t), stream);
