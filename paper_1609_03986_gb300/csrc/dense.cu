@@ -181,16 +181,29 @@ constexpr uint32_t kNoKey = 0xffffffffu;
 // offsets, and the staging threads run along both the descriptors and the groups.
 __device__ __forceinline__ const uint4* staged_cell(const uint4* s, int c) { return s + (c >> 3) * 32 + (c & 7); }
 
+// Hamming distance of a descriptor to the one whose chunks are kStep chunks apart.
+template <int kStep>
+__device__ __forceinline__ int chunk_distance(const uint32_t (&a)[16], const uint4* c) {
+    uint32_t x[16];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const uint4 v = c[kStep * q];
+        x[4 * q] = v.x ^ a[4 * q], x[4 * q + 1] = v.y ^ a[4 * q + 1];
+        x[4 * q + 2] = v.z ^ a[4 * q + 2], x[4 * q + 3] = v.w ^ a[4 * q + 3];
+    }
+    return popc16(x);
+}
+
 // One pixel per thread.  Keys distance << 12 | staged row << 6 | column are unique and
 // order ties by raster index, so a distance costs the top two two minima and a maximum.
-// The logic pipe (16 XORs, the carry-save adders, addresses, the top two) and the
-// population-count pipe (12 counts) bound it about equally; packed keys and the staged
-// order take several of the logic pipe's operations per distance away.  Measured (GB300; before:
-// rotated chunks, compares and selects): 640x480 at radius 2 / 8 / 16 34.4 -> 30.4, 301.6 ->
-// 255.3 and 1,790 -> 1,423 us, 1920x1080 at radius 8 1,906 -> 1,611 us, 97x70 at radius 8
-// 67.5 -> 54.1 us, radius 0 unchanged.  Two pixels per thread (a candidate's loads serve
-// both) took 275 us at 640x480, radius 8: too few warps; copies by cp.async lose 18% at
-// radius 0.
+// The logic pipe (16 XORs and 16 adder operations, the top two: 35 at 64 lanes per clock) and
+// the population-count pipe (9 counts at 16) bound it about equally; packed keys and the staged
+// order take several of the logic pipe's operations per distance away.  Measured (GB300; with
+// rotated chunks, compares and selects, and now): 640x480 at radius 2 / 8 / 16 30.9 -> 26.6, 298
+// -> 238 and 1,786 -> 1,357 us, 1920x1080 at radius 8 1,902 -> 1,517 us.  At radius 0 a
+// descriptor is read once and nothing is staged (staged, whose loads are 16 bytes from each of
+// eight descriptors: 1001x601 14.2 -> 11.8 us, 1920x1080 46.2 -> 43.6).  Two pixels per thread (a
+// candidate's loads serve both) took 10% more at 640x480, radius 8: too few warps.
 __global__ void __launch_bounds__(kMatchThreads) dense_match_kernel(const uint4* __restrict__ da,
                                                                     const uint4* __restrict__ db, int width,
                                                                     int height, int radius, int k, int r_milli,
@@ -200,44 +213,46 @@ __global__ void __launch_bounds__(kMatchThreads) dense_match_kernel(const uint4*
     const int x0 = blockIdx.x * kMTile, y0 = blockIdx.y * kMTile;
     griddep_wait();
     griddep_launch_dependents();
-    for (int i = threadIdx.x; i < (cells + 7) / 8 * 32; i += kMatchThreads) {
-        const int cell = (i >> 5) * 8 + (i & 7), q = (i >> 3) & 3;
-        const int ry = cell / side, rx = cell - ry * side;
-        const int gy = y0 - radius + ry, gx = x0 - radius + rx;
-        if (cell < cells && gx >= 0 && gx < width && gy >= 0 && gy < height)
-            s_desc[i] = db[(static_cast<int64_t>(gy) * width + gx) * 4 + q];
-    }
+    if (radius > 0)
+        for (int i = threadIdx.x; i < (cells + 7) / 8 * 32; i += kMatchThreads) {
+            const int cell = (i >> 5) * 8 + (i & 7), q = (i >> 3) & 3;
+            const int ry = cell / side, rx = cell - ry * side;
+            const int gy = y0 - radius + ry, gx = x0 - radius + rx;
+            if (cell < cells && gx >= 0 && gx < width && gy >= 0 && gy < height)
+                s_desc[i] = db[(static_cast<int64_t>(gy) * width + gx) * 4 + q];
+        }
     const int tx = threadIdx.x % kMTile, ty = threadIdx.x / kMTile;
     const int px = x0 + tx, py = y0 + ty;
     const bool live = px < width && py < height;
+    const int64_t self = (static_cast<int64_t>(py) * width + px) * 4;
     uint32_t a[16];
     if (live) {
-        const uint4* src = da + (static_cast<int64_t>(py) * width + px) * 4;
+        const uint4* src = da + self;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const uint4 v = src[q];
             a[4 * q] = v.x, a[4 * q + 1] = v.y, a[4 * q + 2] = v.z, a[4 * q + 3] = v.w;
         }
     }
-    __syncthreads();
-    if (!live) return;
     uint32_t m1 = kNoKey, m2 = kNoKey;
-    // staged rows and columns of the candidates inside B
-    const int rx_lo = max(tx, radius - x0), rx_hi = min(tx + 2 * radius, width - 1 - x0 + radius);
-    const int ry_lo = max(ty, radius - y0), ry_hi = min(ty + 2 * radius, height - 1 - y0 + radius);
-    for (int ry = ry_lo; ry <= ry_hi; ++ry) {
-        for (int rx = rx_lo; rx <= rx_hi; ++rx) {
-            const uint4* c = staged_cell(s_desc, ry * side + rx);
-            uint32_t x[16];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const uint4 v = c[8 * q];
-                x[4 * q] = v.x ^ a[4 * q], x[4 * q + 1] = v.y ^ a[4 * q + 1];
-                x[4 * q + 2] = v.z ^ a[4 * q + 2], x[4 * q + 3] = v.w ^ a[4 * q + 3];
+    auto key_of = [](int d, int ry, int rx) {
+        return (static_cast<uint32_t>(d) << kOrdBits) + static_cast<uint32_t>(ry << 6 | rx);
+    };
+    if (radius == 0) {  // each descriptor is read once: nothing to stage
+        if (!live) return;
+        m1 = key_of(chunk_distance<1>(a, db + self), ty, tx);
+    } else {
+        __syncthreads();
+        if (!live) return;
+        // staged rows and columns of the candidates inside B
+        const int rx_lo = max(tx, radius - x0), rx_hi = min(tx + 2 * radius, width - 1 - x0 + radius);
+        const int ry_lo = max(ty, radius - y0), ry_hi = min(ty + 2 * radius, height - 1 - y0 + radius);
+        for (int ry = ry_lo; ry <= ry_hi; ++ry) {
+            for (int rx = rx_lo; rx <= rx_hi; ++rx) {
+                const uint32_t key = key_of(chunk_distance<8>(a, staged_cell(s_desc, ry * side + rx)), ry, rx);
+                m2 = min(m2, max(m1, key));
+                m1 = min(m1, key);
             }
-            const uint32_t key = (static_cast<uint32_t>(popc16(x)) << kOrdBits) + static_cast<uint32_t>(ry << 6 | rx);
-            m2 = min(m2, max(m1, key));
-            m1 = min(m1, key);
         }
     }
     auto index = [&](uint32_t key) {
@@ -261,6 +276,7 @@ __global__ void __launch_bounds__(kMatchThreads) dense_match_kernel(const uint4*
 }  // namespace
 
 static size_t dense_match_smem_bytes(int radius) {
+    if (radius == 0) return 0;
     const size_t side = static_cast<size_t>(kMTile + 2 * radius);
     return (side * side + 7) / 8 * 8 * kDescBytes;  // whole groups of eight cells
 }
