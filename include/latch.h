@@ -144,7 +144,8 @@ latch_status latch_set_triplets(latch_context *ctx, const latch_triplet *h_tripl
 latch_status latch_set_patch_weights(latch_context *ctx, const uint8_t *h_weights);
 
 /* Pre-size the context's scratch memory so that later calls up to these sizes
- * allocate nothing (required before capturing calls in a CUDA graph). */
+ * allocate nothing (required before capturing calls in a CUDA graph).  Extraction needs
+ * no scratch: max_keypoints is only checked. */
 latch_status latch_reserve(latch_context *ctx, int64_t max_keypoints, int64_t max_query, int64_t max_train);
 
 /*

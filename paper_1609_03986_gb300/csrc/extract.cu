@@ -1014,23 +1014,6 @@ void plan_triplets(const latch_triplet* trip, int size, LaneTripletPlan* plan) {
     }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static EncodeTiledFn extract_encode_fn() {
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(p);
-    }
-    return fn;
-}
-
 static constexpr int kBatchImages = 64;  // images per launch in the batched form
 static_assert(sizeof(ExtractParams<kBatchImages>) + sizeof(LaneTriplets) + sizeof(PatchWeights) + 64 <= 32764,
               "kernel parameter space");
@@ -1049,7 +1032,7 @@ static cudaError_t launch_chunk(const latch_context* ctx, const latch_image* img
     cudaError_t e = ctx->weighted ? once_per_device(&attr_done[1], set_extract_attributes<NI, true>)
                                   : once_per_device(&attr_done[0], set_extract_attributes<NI, false>);
     if (e != cudaSuccess) return e;
-    EncodeTiledFn enc = extract_encode_fn();
+    const EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return cudaErrorNotSupported;
     struct Params {
         ExtractParams<NI> prm;
