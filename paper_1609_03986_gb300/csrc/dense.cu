@@ -63,6 +63,8 @@ struct DenseSmem {
     alignas(16) int32_t h[2][2][kHRows][kHPitch];  // [round parity][triplet slot][row][column]
 };
 
+// Three blocks per SM at 64 registers (24 bytes spilled); launch bounds of
+// four and five blocks spill more and are slower.
 __global__ void __launch_bounds__(kDenseThreads, 3) dense_extract_kernel(const uint8_t* __restrict__ img, int width,
                                                                       int height, int64_t pitch, int half,
                                                                       const __grid_constant__ DenseTriplets tr,

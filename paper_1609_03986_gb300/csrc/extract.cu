@@ -17,9 +17,9 @@
 //   16 evaluators  first copy the batch's staged words into tensor memory, window j in
 //                  TMEM lane j of every lane quarter, and evaluate the triplets that no
 //                  quarter holds from the staged windows, which frees the staging buffer
-//                  for the next batch; then evaluate the others by Eq. 1, all 32 lanes on the same triplet:
-//                  a patch is two or three columns of words, so as many 8-row TMEM loads
-//                  bring it, its rows are aligned by funnel shifts, and D1 - D2 =
+//                  for the next batch; then evaluate the others by Eq. 1, all 32 lanes on
+//                  the same triplet: a patch is two or three columns of words, so as many
+//                  8-row TMEM loads bring it, its rows are aligned by funnel shifts, and D1 - D2 =
 //                  (sum C1^2 - sum C2^2) - 2 (sum A.C1 - sum A.C2) by __dp4a, all exact in
 //                  32-bit integers.  A ballot gives a triplet's bit of all 32 keypoints;
 //                  the bits are transposed and leave as whole rows, with the tensor
@@ -32,9 +32,11 @@
 // windows.  512 columns hold 504 of a window's 576 words.  As all four quarters hold the
 // same keypoints, each keeps another part of the window, from another byte of a word on,
 // and a triplet is evaluated in a quarter that holds its patches, where most of them start
-// at a word and need no alignment (25 of 42 shifts are left on the seeded table).  The
-// evaluation is bound by instruction issue (about 125 instructions per triplet, 56 of
-// them dot products) shared with the builders.
+// at a word and need no alignment (25 of 42 shifts are left on the seeded table).
+// Instruction issue bounds the kernel: the evaluation's 125 instructions per triplet (56 of
+// them dot products) are half of what a keypoint takes, sampling and copying its window, the
+// waits and the output the other half.  The four quarters are the four partitions of an SM:
+// plan_triplets levels them (to 0.2% of its own costs on the seeded table).
 //
 // Why a tile per keypoint: no sort by image cell is needed (it cost a memset and two
 // launches in front of the extraction), builders need no barrier between keypoints, and at
@@ -46,8 +48,8 @@
 // the same result and raises the context's device flag.
 //
 // Measured (GB300, whole calls back to back; before: windows in shared memory, cell sort):
-// 257 keypoints of 321x243 46.9 -> 18.4 us, 2,000 of 640x480 44.1 -> 22.7 us, 10,000 of
-// 1920x1080 91.4 -> 52.8 us, the same weighted 189 -> 134 us.
+// 257 keypoints of 321x243 47.2 -> 18.2 us, 2,000 of 640x480 45.2 -> 21.0 us, 10,000 of
+// 1920x1080 92.2 -> 50.8 us, the same weighted 190 -> 124 us.
 #include <cuda.h>
 
 #include <cmath>

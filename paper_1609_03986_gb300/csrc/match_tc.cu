@@ -51,10 +51,10 @@
 // K = 96 they are no faster than 846 because of the operand reads).  In a pair each block
 // reads its own query rows but only half of the train rows, and copies half: 94 KB, 735
 // clocks, next to 720 of MMAs (K = 96 issues 1.5 times the products of K = 64 per clock).
-// Measured (GB300, before: single blocks, K = 64, an MMA thread of its own): 16,384 x
-// 1,048,576 descriptors 2,386 -> 1,783 us (943 clocks per unit), 10,000 x 10,000 46.3 ->
-// 43.4 us, a batch of 64 images and 476 pairs (3.4e11 distances) 59.8 -> 52.4 ms.  What is
-// left above 720 clocks is the accumulators' round trip (MMA end, commit, TMEM loads of 20
+// Measured (GB300, whole calls; single blocks, K = 64 and an MMA thread of its own, and now):
+// 16,384 x 1,048,576 descriptors 2,369 -> 1,768 us (about 945 clocks per unit), 10,000 x 10,000
+// 46.4 -> 42.0 us, a batch of 64 images and 476 pairs (3.4e11 distances, extraction included)
+// 67.0 -> 51.1 ms.  What is left above 720 clocks is the accumulators' round trip (MMA end, commit, TMEM loads of 20
 // warps, arrivals of both blocks, next MMA: about 1,200 clocks for two accumulators in
 // flight); three accumulators of 160 columns are slower (2,357 us: the epilogue's time per
 // unit hardly depends on its columns).  Short walks are bound by the top-two updates of
@@ -728,8 +728,7 @@ __global__ void expand_kernel(const uint32_t* __restrict__ in, int64_t nwords, u
 
 // The same for a single problem: the query set, then the train set behind it, and the
 // matcher's arrival counters and row bounds cleared, in one launch.  (Two expansions and a memset in
-// front of the matcher cost about 2 us more: 10,000 x 10,000 descriptors match in 45
-// instead of 47 us.)
+// front of the matcher cost about 2 us more.)
 __global__ void expand_two_kernel(const uint32_t* __restrict__ q, int64_t qwords, const uint32_t* __restrict__ t,
                                   int64_t twords, uint4* __restrict__ out, int32_t* __restrict__ counters,
                                   int32_t ncounters, int32_t* __restrict__ bounds, int32_t nbounds) {

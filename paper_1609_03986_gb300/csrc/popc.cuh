@@ -27,7 +27,7 @@ __device__ __forceinline__ void hadd(uint32_t& h, uint32_t& l, uint32_t a, uint3
 // operations and held the population-count pipe (16 lanes per clock against 64) fullest.
 // Measured (GB300, 8 / 9 / 11 words folded): 10,000 x 10,000 on the CUDA cores 339 / 315 /
 // 306 us, 16,384 x 131,072 6,558 / 6,064 / 5,885 us, the dense matcher at 640x480 and
-// radius 8 255 / 246 / 248 us.
+// radius 8 255 / 246 / 248 us (as it was written then; 238 now).
 __device__ __forceinline__ int popc16(const uint32_t (&x)[16]) {
     uint32_t h0, h1, h2, h3, h4, l0, l1, l2, l3, ones;
     csa(h0, l0, x[0], x[1], x[2]);
