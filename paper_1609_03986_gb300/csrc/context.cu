@@ -121,7 +121,7 @@ static latch_status upload_scales(latch_context* ctx, const double* scales, int 
 // walks a unit of the same query tile and the last one combines 60 to 76 records a row (1 x
 // 20,000: 30.9 / 36.7, 6 x 30,000 35.0 / 37.8, 8 x 24,000 35.2 / 37.4; about equal at 8 x 28,000
 // and 12 x 24,000; 4 x 34,000 40.1 / 38.1, 16 x 26,000 39.1 / 37.4).  Beyond 65,536 rows the pair
-// count decides alone, although the tensor cores are faster there too (30 x 140,000 309 / 51):
+// count decides alone, although the tensor cores are faster there too (16 x 100,000 214 / 47):
 // the path's scratch is 256 bytes per row, and the context keeps it -- a gigabyte for a single
 // query against 2^22 rows, which such a call never took.
 bool small_problem_to_tensor(int64_t nq, int64_t nt) {
